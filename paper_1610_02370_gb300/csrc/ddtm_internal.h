@@ -235,7 +235,10 @@ void launch_dslash_multi(const FineGeom& g, int prec, void* y, float* ynrm, cons
                          const void* links, const void* clover, double mu, int nrhs, cudaStream_t s);
 
 // ---- sap.cu ----------------------------------------------------------------------
-void launch_sap_half(const FineGeom& g, int prec, void* x, float* xn, const void* b, const float* bn, const void* links,
+// blocks of 4^4 sites: FP16 fields may take the operator (links, clover, sinv) in precision po = F32;
+// po = prec otherwise
+bool sap_b4_blocks(const FineGeom& g);
+void launch_sap_half(const FineGeom& g, int prec, int po, void* x, float* xn, const void* b, const float* bn, const void* links,
                      const void* clover, const void* sinv, const int* blocks, const int* zero_blocks, int nblocks,
                      int zero_x, int nmr, double mu, int nrhs, cudaStream_t s);
 

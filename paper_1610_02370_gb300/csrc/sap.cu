@@ -21,6 +21,7 @@
 #include "ddtm_internal.h"
 #include "timer.h"
 #include "stencil.cuh"
+#include "stencil_lanes.cuh"
 
 namespace ddtm {
 
@@ -222,6 +223,420 @@ __global__ void __launch_bounds__(128 * RG, P == PREC_F64 ? 2 : 4 / RG)
   }
 }
 
+// ---- 4^4 blocks, FP32 arithmetic ---------------------------------------------------
+// The same half-sweep, one CTA per block and right-hand side (V = float, k_sap_half_b4_one) or pair of
+// right-hand sides (V = float2, k_sap_half_b4).  The correction of the even sites is accumulated as
+//   e_e = A_ee^-1 r_e - sum_k alpha_k A_ee^-1 A_eo rho_k,
+// whose terms the MR steps form anyway, so the closing hop and inverse of step 4 above are not needed.
+// Shared memory: bufE, bufO (the vectors the hops read) and accE, accO, 12 x 128 complex each.
+// Both kernels form every sum in the same order (forward hops, backward hops, their sum; inner products per
+// chirality and warp, then over the eight of them), so a right-hand side gets the same bits from either.
+//
+// What bounds them (24^3 x 48, 12 right-hand sides, FP16 fields, one cycle of 3 MR steps: 2.77 ms, before
+// 5.85 ms with k_sap_half; one right-hand side 0.34 ms, before 0.63 ms): the shared-memory data path (about
+// 0.8 ms per half-sweep of spinor and operator reads) and, with 8 warps per SM for the pair, the latency of the
+// operator reads from L2.  Packing two right-hand sides cut the instructions from 2.17 G to 0.71 G per half-sweep.
+// Measured and not taken for the pair: accE and accO in local memory for more warps per SM (3.07 ms with 2 CTAs, 3.01
+// with 3, 3.66 with 4 per SM), two pairs per CTA (2.96 ms: their phases coincide), two threads per site as below
+// (2.97 ms: 128 registers spill), the faces of the residual staged in shared memory first (2.68 ms, no gain).
+template <typename V>
+__host__ __device__ constexpr size_t sap_b4_smem() {
+  return 4 * 12 * B4_VH * sizeof(cv<V>) + 2 * 8 * 3 * sizeof(V);
+}
+
+// partial sums of <p, rho> = sum conj(p) rho (s0 + i s1) and <p, p> (s2) over one chirality
+template <typename V>
+__device__ __forceinline__ void sap_dots(const cv<V> p[6], const cv<V> r[6], V& s0, V& s1, V& s2) {
+  s0 = s1 = s2 = vset<V>(0.f);
+#pragma unroll
+  for (int c = 0; c < 6; c++) {
+    s0 = vfma(p[c].re, r[c].re, vfma(p[c].im, r[c].im, s0));
+    s1 = vsub(vfma(p[c].re, r[c].im, s1), vmul(p[c].im, r[c].re));
+    s2 = vfma(p[c].re, p[c].re, vfma(p[c].im, p[c].im, s2));
+  }
+#pragma unroll
+  for (int l = 0; l < vlanes<V>(); l++) {
+    const float t0 = warp_sum(vlane(s0, l)), t1 = warp_sum(vlane(s1, l)), t2 = warp_sum(vlane(s2, l));
+    vput(s0, l, t0);
+    vput(s1, l, t1);
+    vput(s2, l, t2);
+  }
+}
+// alpha = <p, rho> / <p, p> from the eight partial sums
+template <typename V> __device__ __forceinline__ void sap_alpha(const V* rd, V& are, V& aim) {
+  V s0 = vset<V>(0.f), s1 = s0, s2 = s0;
+#pragma unroll
+  for (int w = 0; w < 8; w++) {
+    s0 = vadd(s0, rd[3 * w]);
+    s1 = vadd(s1, rd[3 * w + 1]);
+    s2 = vadd(s2, rd[3 * w + 2]);
+  }
+#pragma unroll
+  for (int l = 0; l < vlanes<V>(); l++) {
+    const float pp = vlane(s2, l);
+    vput(are, l, pp > 0.f ? vlane(s0, l) / pp : 0.f);
+    vput(aim, l, pp > 0.f ? vlane(s1, l) / pp : 0.f);
+  }
+}
+// e_o += alpha rho, e_e -= alpha A_ee^-1 A_eo rho, rho -= alpha p for one chirality at slots o, o + 128, ...
+template <typename V>
+__device__ __forceinline__ void sap_update(cv<V>* accO, cv<V>* accE, cv<V>* bufO, const cv<V>* bufE, int o, V are, V aim,
+                                           const cv<V> r[6], const cv<V> p[6]) {
+  const V nre = vsub(vset<V>(0.f), are), nim = vsub(vset<V>(0.f), aim);
+#pragma unroll
+  for (int c = 0; c < 6; c++, o += B4_VH) {
+    cv<V> e = accO[o], t = bufE[o], f = accE[o], q = r[c];
+    e.re = vfma(are, q.re, vfma(nim, q.im, e.re));
+    e.im = vfma(are, q.im, vfma(aim, q.re, e.im));
+    f.re = vfma(nre, t.re, vfma(aim, t.im, f.re));
+    f.im = vfma(nre, t.im, vfma(nim, t.re, f.im));
+    q.re = vfma(nre, p[c].re, vfma(aim, p[c].im, q.re));
+    q.im = vfma(nre, p[c].im, vfma(nim, p[c].re, q.im));
+    accO[o] = e;
+    accE[o] = f;
+    bufO[o] = q;
+  }
+}
+// r = b - D x at site i of parity par, from the staged x (own, oth: its two parities) into out
+template <int P, int PO, typename V, typename SO>
+__device__ __forceinline__ void sap_residual(cv<V>* out, const cv<V>* own, const cv<V>* oth, const LaneField<P, V>& x,
+                                             const LaneField<P, V>& b, const SO* __restrict__ U, const SO* __restrict__ C,
+                                             const Geo& g, float mu, int blk, int i, int par) {
+  cv<V> acc[12], v[12], s[12];
+  v_hops_full<P, PO>(oth, x, U, g, blk, i, par, acc);
+#pragma unroll
+  for (int c = 0; c < 12; c++) v[c] = own[c * B4_VH + i];
+  v_clover<PO, B4_VB>(C + (size_t)blk * 36 * B4_VB + par * B4_VH + i, v, s);
+  v_twist(mu, v, s);
+  b.load(blk, par * B4_VH + i, v);
+#pragma unroll
+  for (int c = 0; c < 12; c++) {
+    cv<V> o;
+    o.re = vsub(vfma(vset<V>(0.5f), acc[c].re, v[c].re), s[c].re);
+    o.im = vsub(vfma(vset<V>(0.5f), acc[c].im, v[c].im), s[c].im);
+    out[c * B4_VH + i] = o;
+  }
+}
+// x = e (zero_x) or x + e at site i of parity par
+template <int P, typename V>
+__device__ __forceinline__ void sap_store(const LaneField<P, V>& x, const cv<V>* e, int blk, int i, int par, int zero_x, int r0,
+                                          int nrhs) {
+  cv<V> v[12];
+  if (zero_x) {
+#pragma unroll
+    for (int c = 0; c < 12; c++) v[c] = e[c * B4_VH + i];
+  } else {
+    x.load(blk, par * B4_VH + i, v);
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+      const cv<V> q = e[c * B4_VH + i];
+      v[c].re = vadd(v[c].re, q.re);
+      v[c].im = vadd(v[c].im, q.im);
+    }
+  }
+  x.store(blk, par * B4_VH + i, v, r0, nrhs);
+}
+
+// Two right-hand sides: one thread per pair of sites (even i, odd i).
+template <int P, int PO, typename V>
+__global__ void __launch_bounds__(128, 2)
+    k_sap_half_b4(Spinor<P> xf, Spinor<P> bf, const typename Prec<PO>::store2* __restrict__ U,
+                  const typename Prec<PO>::store2* __restrict__ C, const typename Prec<PO>::store2* __restrict__ Ainv,
+                  Geo g, SapArgs<float> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cv<V>* bufE = reinterpret_cast<cv<V>*>(smem_raw);
+  cv<V>* bufO = bufE + 12 * B4_VH;
+  cv<V>* accE = bufO + 12 * B4_VH;
+  cv<V>* accO = accE + 12 * B4_VH;
+  V* red = reinterpret_cast<V*>(accO + 12 * B4_VH);  // [2][2 chiralities][4 warps][3]
+  const int i = threadIdx.x, r0 = blockIdx.x * vlanes<V>();
+  const int blk = a.blocks[blockIdx.y];
+  const LaneField<P, V> x(xf, r0, a.nrhs, a.fstride, a.V), b(bf, r0, a.nrhs, a.fstride, a.V);
+  const typename Prec<PO>::store2* ub = U + (size_t)blk * 36 * B4_VB;
+  const typename Prec<PO>::store2* cb = C + (size_t)blk * 36 * B4_VB + B4_VH + i;
+  const typename Prec<PO>::store2* ib = Ainv + (size_t)blk * 72 * B4_VH + i;
+
+  // block residual on both parities, into accE and accO
+  if (a.zero_x) {
+    const int zb = a.zero_blocks[blockIdx.y];  // one block of the other colour is cleared per CTA
+    cv<V> v[12];
+#pragma unroll
+    for (int c = 0; c < 12; c++) v[c].re = v[c].im = vset<V>(0.f);
+    x.store(zb, i, v, r0, a.nrhs);
+    x.store(zb, B4_VH + i, v, r0, a.nrhs);
+    b.load(blk, i, v);
+#pragma unroll
+    for (int c = 0; c < 12; c++) accE[c * B4_VH + i] = v[c];
+    b.load(blk, B4_VH + i, v);
+#pragma unroll
+    for (int c = 0; c < 12; c++) accO[c * B4_VH + i] = v[c];
+  } else {
+    {
+      cv<V> v[12];
+      x.load(blk, i, v);
+#pragma unroll
+      for (int c = 0; c < 12; c++) bufE[c * B4_VH + i] = v[c];
+      x.load(blk, B4_VH + i, v);
+#pragma unroll
+      for (int c = 0; c < 12; c++) bufO[c * B4_VH + i] = v[c];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int par = 0; par < 2; par++)
+      sap_residual<P, PO>(par ? accO : accE, par ? bufO : bufE, par ? bufE : bufO, x, b, U, C, g, a.mu, blk, i, par);
+    __syncthreads();  // the reads of bufE and bufO are done
+  }
+  // step 0: bufE = A_ee^-1 r_e, rho = bufO = r_o - A_oe bufE; steps 1 ... nmr: minimal residual
+#pragma unroll 1
+  for (int k = 0; k <= a.nmr; k++) {
+    {
+      cv<V> h[12], t[12];
+      if (k == 0) {
+#pragma unroll
+        for (int c = 0; c < 12; c++) h[c] = accE[c * B4_VH + i];
+      } else {
+        cv<V> q[12];
+        v_hops_inside<PO, true>(bufO, ub, i, 0, h);
+        v_hops_inside<PO, false>(bufO, ub, i, 0, q);
+#pragma unroll
+        for (int c = 0; c < 12; c++) {
+          h[c].re = vmul(vset<V>(-0.5f), vadd(h[c].re, q[c].re));
+          h[c].im = vmul(vset<V>(-0.5f), vadd(h[c].im, q[c].im));
+        }
+      }
+      v_site_inv_half<PO, B4_VH>(ib, h, t);
+      v_site_inv_half<PO, B4_VH>(ib + 36 * B4_VH, h + 6, t + 6);
+#pragma unroll
+      for (int c = 0; c < 12; c++) {
+        bufE[c * B4_VH + i] = t[c];
+        if (k == 0) accE[c * B4_VH + i] = t[c];
+      }
+    }
+    __syncthreads();
+    cv<V> h[12];
+    {
+      cv<V> q[12];
+      v_hops_inside<PO, true>(bufE, ub, i, 1, h);
+      v_hops_inside<PO, false>(bufE, ub, i, 1, q);
+#pragma unroll
+      for (int c = 0; c < 12; c++) {
+        h[c].re = vadd(h[c].re, q[c].re);
+        h[c].im = vadd(h[c].im, q[c].im);
+      }
+    }
+    if (k == 0) {
+#pragma unroll
+      for (int c = 0; c < 12; c++) {
+        cv<V> r = accO[c * B4_VH + i];
+        r.re = vfma(vset<V>(0.5f), h[c].re, r.re);
+        r.im = vfma(vset<V>(0.5f), h[c].im, r.im);
+        bufO[c * B4_VH + i] = r;
+        r.re = r.im = vset<V>(0.f);
+        accO[c * B4_VH + i] = r;
+      }
+      __syncthreads();
+      continue;
+    }
+    cv<V> r[12], p[12];
+#pragma unroll
+    for (int c = 0; c < 12; c++) r[c] = bufO[c * B4_VH + i];
+    v_clover<PO, B4_VB>(cb, r, p);
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+      const float mu = c < 6 ? a.mu : -a.mu;
+      p[c].re = vfma(vset<V>(-mu), r[c].im, vfma(vset<V>(0.5f), h[c].re, p[c].re));
+      p[c].im = vfma(vset<V>(mu), r[c].re, vfma(vset<V>(0.5f), h[c].im, p[c].im));
+    }
+    V* rd = red + (k & 1) * 24;
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+      V s0, s1, s2;
+      sap_dots(p + 6 * q, r + 6 * q, s0, s1, s2);
+      if ((i & 31) == 0) {
+        const int w = 4 * q + (i >> 5);
+        rd[3 * w] = s0;
+        rd[3 * w + 1] = s1;
+        rd[3 * w + 2] = s2;
+      }
+    }
+    __syncthreads();
+    V are, aim;
+    sap_alpha(rd, are, aim);
+    sap_update(accO, accE, bufO, bufE, i, are, aim, r, p);
+    sap_update(accO, accE, bufO, bufE, 6 * B4_VH + i, are, aim, r + 6, p + 6);
+    __syncthreads();
+  }
+#pragma unroll 1
+  for (int par = 0; par < 2; par++) sap_store(x, par ? accO : accE, blk, i, par, a.zero_x, r0, a.nrhs);
+}
+
+// One right-hand side, where latency counts: 256 threads.  The residual takes one thread per site; in the
+// block solve two threads share a site, the first (half 0) sums the forward hops, the second the backward
+// hops, they exchange the chirality the other one owns, and each goes on with its own chirality
+// (inverse, clover, minimal-residual update).
+template <int P, int PO, typename V>
+__global__ void __launch_bounds__(256, 2)
+    k_sap_half_b4_one(Spinor<P> xf, Spinor<P> bf, const typename Prec<PO>::store2* __restrict__ U,
+                      const typename Prec<PO>::store2* __restrict__ C, const typename Prec<PO>::store2* __restrict__ Ainv,
+                      Geo g, SapArgs<float> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cv<V>* bufE = reinterpret_cast<cv<V>*>(smem_raw);
+  cv<V>* bufO = bufE + 12 * B4_VH;
+  cv<V>* accE = bufO + 12 * B4_VH;
+  cv<V>* accO = accE + 12 * B4_VH;
+  V* red = reinterpret_cast<V*>(accO + 12 * B4_VH);  // [2][8 warps][3]
+  const int hf = threadIdx.x >> 7, i = threadIdx.x & 127, r0 = blockIdx.x * vlanes<V>();
+  const int blk = a.blocks[blockIdx.y];
+  const typename Prec<PO>::store2* ub = U + (size_t)blk * 36 * B4_VB;
+
+  const LaneField<P, V> x(xf, r0, a.nrhs, a.fstride, a.V);
+  // block residual, thread = site (half = parity), into accE and accO
+  {
+    const LaneField<P, V> b(bf, r0, a.nrhs, a.fstride, a.V);
+    cv<V>* out = hf ? accO : accE;
+    cv<V> v[12];
+    if (a.zero_x) {
+#pragma unroll
+      for (int c = 0; c < 12; c++) v[c].re = v[c].im = vset<V>(0.f);
+      x.store(a.zero_blocks[blockIdx.y], threadIdx.x, v, r0, a.nrhs);  // clear one block of the other colour
+      b.load(blk, threadIdx.x, v);
+#pragma unroll
+      for (int c = 0; c < 12; c++) out[c * B4_VH + i] = v[c];
+    } else {
+      cv<V>* own = hf ? bufO : bufE;
+      x.load(blk, threadIdx.x, v);
+#pragma unroll
+      for (int c = 0; c < 12; c++) own[c * B4_VH + i] = v[c];
+      __syncthreads();
+      sap_residual<P, PO>(out, own, hf ? bufE : bufO, x, b, U, C, g, a.mu, blk, i, hf);
+    }
+    __syncthreads();
+  }
+  const int o0 = 6 * hf * B4_VH + i, x0 = 6 * (hf ^ 1) * B4_VH + i;  // own chirality, the other one
+  const typename Prec<PO>::store2* cb = C + ((size_t)blk * 36 + 18 * hf) * B4_VB + B4_VH + i;
+  const typename Prec<PO>::store2* ib = Ainv + ((size_t)blk * 72 + 36 * hf) * B4_VH + i;
+  const float mu = hf ? -a.mu : a.mu;
+  // phases 0, 1: bufE = A_ee^-1 r_e, rho = bufO = r_o - A_oe bufE; phases 2 k, 2 k + 1: MR step k
+#pragma unroll 1
+  for (int ph = 0; ph < 2 * a.nmr + 2; ph++) {
+    const int par = ph & 1;
+    cv<V>* dst = par ? bufO : bufE;
+    cv<V> r[6], h[6];
+    if (ph == 0) {
+#pragma unroll
+      for (int c = 0; c < 6; c++) h[c] = accE[o0 + c * B4_VH];
+    } else {
+      cv<V> acc[12];
+      if (par)
+#pragma unroll
+        for (int c = 0; c < 6; c++) r[c] = (ph == 1 ? accO : bufO)[o0 + c * B4_VH];
+      // partial sums of the other chirality go to its owner: in an odd phase through the slots of bufO whose
+      // entries are now in r, in an even phase through slots of bufE, whose entries are no longer needed
+      cv<V>* put = dst + (par ? o0 : x0);
+      const cv<V>* get = dst + (par ? x0 : o0);
+      if (hf == 0) {
+        v_hops_inside<PO, true>(par ? bufE : bufO, ub, i, par, acc);
+#pragma unroll
+        for (int c = 0; c < 6; c++) put[c * B4_VH] = acc[6 + c];
+#pragma unroll
+        for (int c = 0; c < 6; c++) h[c] = acc[c];
+      } else {
+        v_hops_inside<PO, false>(par ? bufE : bufO, ub, i, par, acc);
+#pragma unroll
+        for (int c = 0; c < 6; c++) put[c * B4_VH] = acc[c];
+#pragma unroll
+        for (int c = 0; c < 6; c++) h[c] = acc[6 + c];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < 6; c++) {
+        const cv<V> q = get[c * B4_VH];
+        h[c].re = vadd(h[c].re, q.re);
+        h[c].im = vadd(h[c].im, q.im);
+      }
+    }
+    if (par == 0) {  // bufE = A_ee^-1 h, h = r_e or H_eo rho
+      cv<V> t[6];
+      if (ph)
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+          h[c].re = vmul(vset<V>(-0.5f), h[c].re);
+          h[c].im = vmul(vset<V>(-0.5f), h[c].im);
+        }
+      v_site_inv_half<PO, B4_VH>(ib, h, t);
+#pragma unroll
+      for (int c = 0; c < 6; c++) {
+        bufE[o0 + c * B4_VH] = t[c];
+        if (ph == 0) accE[o0 + c * B4_VH] = t[c];
+      }
+      __syncthreads();
+      continue;
+    }
+    if (ph == 1) {
+      __syncthreads();  // the exchanged sums are read
+#pragma unroll
+      for (int c = 0; c < 6; c++) {
+        r[c].re = vfma(vset<V>(0.5f), h[c].re, r[c].re);
+        r[c].im = vfma(vset<V>(0.5f), h[c].im, r[c].im);
+        bufO[o0 + c * B4_VH] = r[c];
+        r[c].re = r[c].im = vset<V>(0.f);
+        accO[o0 + c * B4_VH] = r[c];
+      }
+      __syncthreads();
+      continue;
+    }
+    cv<V> p[6];
+    v_clover_half<PO, B4_VB>(cb, r, p);
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+      p[c].re = vfma(vset<V>(-mu), r[c].im, vfma(vset<V>(0.5f), h[c].re, p[c].re));
+      p[c].im = vfma(vset<V>(mu), r[c].re, vfma(vset<V>(0.5f), h[c].im, p[c].im));
+    }
+    V s0, s1, s2;
+    sap_dots(p, r, s0, s1, s2);
+    V* rd = red + (ph & 2) * 12;  // alternates from step to step
+    if ((i & 31) == 0) {
+      const int w = threadIdx.x >> 5;
+      rd[3 * w] = s0;
+      rd[3 * w + 1] = s1;
+      rd[3 * w + 2] = s2;
+    }
+    __syncthreads();
+    V are, aim;
+    sap_alpha(rd, are, aim);
+    sap_update(accO, accE, bufO, bufE, o0, are, aim, r, p);
+    __syncthreads();
+  }
+  sap_store(x, hf ? accO : accE, blk, i, hf, a.zero_x, r0, a.nrhs);
+}
+
+template <int P, int PO>
+static void launch_sap_b4(const FineGeom& g, void* x, float* xn, const void* b, const float* bn, const void* links,
+                          const void* clover, const void* sinv, const int* blocks, const int* zero_blocks, int nblocks,
+                          int zero_x, int nmr, double mu, int nrhs, cudaStream_t s) {
+  typedef typename Prec<P>::store2 S;
+  typedef typename Prec<PO>::store2 SO;
+  Geo q{g.Vb, g.Nb, g.loc_nbr.as<uint32_t>(), g.blk_nbr.as<int>()};
+  const bool two = nrhs > 1;
+  const void* kern = two ? (const void*)k_sap_half_b4<P, PO, float2> : (const void*)k_sap_half_b4_one<P, PO, float>;
+  const size_t smem = two ? sap_b4_smem<float2>() : sap_b4_smem<float>();
+  set_dynamic_smem(kern, smem);
+  const Spinor<P> X{(S*)x, xn, g.Vb}, B{(S*)b, (float*)bn, g.Vb};
+  for (int b0 = 0; b0 < nblocks; b0 += 65535) {  // grid.y, as below
+    const int nb = nblocks - b0 < 65535 ? nblocks - b0 : 65535;
+    SapArgs<float> a{blocks + b0, nrhs, zero_blocks + b0, zero_x, nmr, (float)mu, (size_t)g.V * 12, g.V};
+    if (two)
+      k_sap_half_b4<P, PO, float2><<<dim3((nrhs + 1) / 2, nb), 128, smem, s>>>(X, B, (const SO*)links, (const SO*)clover,
+                                                                             (const SO*)sinv, q, a);
+    else
+      k_sap_half_b4_one<P, PO, float><<<dim3(1, nb), 256, smem, s>>>(X, B, (const SO*)links, (const SO*)clover,
+                                                                    (const SO*)sinv, q, a);
+    CKL("sap_half");
+  }
+}
+
+bool sap_b4_blocks(const FineGeom& g) { return g.b[0] == 4 && g.b[1] == 4 && g.b[2] == 4 && g.b[3] == 4; }
+
 size_t sap_smem_bytes(int Vb, int prec) {
   return prec == PREC_F64 ? sap_group_smem<double>(Vb / 2) : sap_group_smem<float>(Vb / 2);
 }
@@ -271,11 +686,18 @@ static int sap_rhs_groups(const FineGeom& g, int prec, int nrhs) {
 }
 
 template <int P>
-static void launch_sap_half_t(const FineGeom& g, void* x, float* xn, const void* b, const float* bn, const void* links,
+static void launch_sap_half_t(const FineGeom& g, int po, void* x, float* xn, const void* b, const float* bn, const void* links,
                               const void* clover, const void* sinv, const int* blocks, const int* zero_blocks,
                               int nblocks, int zero_x, int nmr, double mu, int nrhs, cudaStream_t s) {
   const int rg = sap_rhs_groups(g, P, nrhs);
   if constexpr (P != PREC_F64) {
+    if (sap_b4_blocks(g)) {
+      if (po == PREC_F32)
+        launch_sap_b4<P, PREC_F32>(g, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
+      else
+        launch_sap_b4<P, P>(g, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
+      return;
+    }
     if (rg == 4) {
       launch_sap_rg<P, 4>(g, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
       return;
@@ -288,16 +710,16 @@ static void launch_sap_half_t(const FineGeom& g, void* x, float* xn, const void*
   launch_sap_rg<P, 1>(g, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
 }
 
-void launch_sap_half(const FineGeom& g, int prec, void* x, float* xn, const void* b, const float* bn, const void* links,
+void launch_sap_half(const FineGeom& g, int prec, int po, void* x, float* xn, const void* b, const float* bn, const void* links,
                      const void* clover, const void* sinv, const int* blocks, const int* zero_blocks, int nblocks,
                      int zero_x, int nmr, double mu, int nrhs, cudaStream_t s) {
   ScopedTimer timer_(prec == PREC_F64 ? "sap_half_f64" : prec == PREC_F32 ? "sap_half_f32" : "sap_half_f16", s, nrhs);
   if (prec == PREC_F64)
-    launch_sap_half_t<PREC_F64>(g, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
+    launch_sap_half_t<PREC_F64>(g, po, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
   else if (prec == PREC_F32)
-    launch_sap_half_t<PREC_F32>(g, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
+    launch_sap_half_t<PREC_F32>(g, po, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
   else
-    launch_sap_half_t<PREC_F16>(g, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
+    launch_sap_half_t<PREC_F16>(g, po, x, xn, b, bn, links, clover, sinv, blocks, zero_blocks, nblocks, zero_x, nmr, mu, nrhs, s);
 }
 
 }  // namespace ddtm
