@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "ddtm_internal.h"
 #include "timer.h"
+#include "stencil_lanes.cuh"
 
 namespace ddtm {
 
@@ -413,6 +414,51 @@ __global__ void __launch_bounds__(VB, 3)
   }
 }
 
+// The same for 4^4 blocks (stencil_lanes.cuh): one CTA per block and right-hand side (V = float) or pair
+// (V = float2), one thread per site.  CTAs are ordered by chunks of blocks, within a chunk pair after
+// pair, so that the operator of a chunk stays in L2 for all the pairs while the neighbour blocks of one
+// pair are still there (chunks of 32 to 128 blocks measured alike; 512 blocks 20 % slower at 24^3 x 48).
+// Measured (L2 warm, FP32 / FP16 storage): 24^3 x 48, 12 right-hand sides 737 / 688 us (k_dslash_blk 1133 /
+// 986), one 104 / 79 us (112 / 100).  One right-hand side in FP32 is bound by HBM (73 % of the measured copy
+// rate); the batch by L2 reads (0.5 MB per CTA, of which the faces take 0.2 because a face in x uses a
+// quarter of each sector) and their latency at 16 warps per SM.  Not taken: 128 threads per block with the two
+// parities in turn (703 / 790, one 118 / 83), the faces staged in shared memory first (1020 / 822), three pairs per CTA
+// sharing the operator through L1 (874 / 834).
+template <int P, typename V>
+__global__ void __launch_bounds__(256, vlanes<V>() == 2 ? 2 : 3)
+    k_dslash_b4(Spinor<P> yf, Spinor<P> xf, const typename Prec<P>::store2* __restrict__ U,
+                const typename Prec<P>::store2* __restrict__ C, Geo g, float mu, int nrhs, size_t fstride, long Vs,
+                int chunk) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cv<V>* xs = reinterpret_cast<cv<V>*>(smem_raw);  // [2 parities][12][128]
+  const int par = threadIdx.x >> 7, i = threadIdx.x & 127, groups = (nrhs + vlanes<V>() - 1) / vlanes<V>();
+  int blk, r0;
+  {
+    const int c0 = (int)(blockIdx.x / (unsigned)(chunk * groups)) * chunk, rem = (int)(blockIdx.x % (unsigned)(chunk * groups));
+    const int n = g.Nb - c0 < chunk ? g.Nb - c0 : chunk;
+    r0 = rem / n * vlanes<V>();
+    blk = c0 + rem % n;
+  }
+  const LaneField<P, V> x(xf, r0, nrhs, fstride, Vs);
+  cv<V> acc[12], v[12], s[12];
+  x.load(blk, threadIdx.x, v);
+#pragma unroll
+  for (int c = 0; c < 12; c++) xs[(par * 12 + c) * B4_VH + i] = v[c];
+  __syncthreads();
+  v_hops_full<P, P>(xs + (par ^ 1) * 12 * B4_VH, x, U, g, blk, i, par, acc);
+#pragma unroll
+  for (int c = 0; c < 12; c++) v[c] = xs[(par * 12 + c) * B4_VH + i];
+  v_clover<P, B4_VB>(C + (size_t)blk * 36 * B4_VB + threadIdx.x, v, s);
+  v_twist(mu, v, s);
+#pragma unroll
+  for (int c = 0; c < 12; c++) {
+    s[c].re = vfma(vset<V>(-0.5f), acc[c].re, s[c].re);
+    s[c].im = vfma(vset<V>(-0.5f), acc[c].im, s[c].im);
+  }
+  const LaneField<P, V> y(yf, r0, nrhs, fstride, Vs);
+  y.store(blk, threadIdx.x, s, r0, nrhs);
+}
+
 static Geo make_geo(const FineGeom& g) {
   Geo q;
   q.Vb = g.Vb;
@@ -425,11 +471,28 @@ static Geo make_geo(const FineGeom& g) {
 // Block kernels exist for 4^4 blocks (VB = 256) in FP32 and FP16 storage.
 static bool dslash_blk_ok(const FineGeom& g, int prec) { return prec != PREC_F64 && g.Vb == 256; }
 
+static const int B4_CHUNK = 64;
+template <int P, typename V>
+static void dslash_b4_t(const FineGeom& g, Spinor<P> Y, Spinor<P> X, const typename Prec<P>::store2* U,
+                        const typename Prec<P>::store2* C, double mu, int nrhs, cudaStream_t s) {
+  const size_t smem = 2 * 12 * B4_VH * sizeof(cv<V>);
+  set_dynamic_smem((const void*)k_dslash_b4<P, V>, smem);
+  const unsigned groups = (nrhs + vlanes<V>() - 1) / vlanes<V>();
+  k_dslash_b4<P, V><<<(unsigned)g.Nb * groups, 256, smem, s>>>(Y, X, U, C, make_geo(g), (float)mu, nrhs,
+                                                              (size_t)g.V * 12, g.V, B4_CHUNK);
+  CKL("dslash_b4");
+}
+
 template <int P>
 static void dslash_blk_t(const FineGeom& g, void* y, float* ynrm, const void* x, const float* xnrm, const void* links,
                          const void* clover, double mu, int nrhs, cudaStream_t s) {
   typedef typename Prec<P>::store2 S;
   Spinor<P> Y{(S*)y, ynrm, g.Vb}, X{(S*)x, (float*)xnrm, g.Vb};
+  if (g.b[0] == 4 && g.b[1] == 4 && g.b[2] == 4 && g.b[3] == 4) {
+    if (nrhs > 1) dslash_b4_t<P, float2>(g, Y, X, (const S*)links, (const S*)clover, mu, nrhs, s);
+    else dslash_b4_t<P, float>(g, Y, X, (const S*)links, (const S*)clover, mu, nrhs, s);
+    return;
+  }
   k_dslash_blk<P, 256><<<g.Nb, 256, 0, s>>>(Y, X, Links<P>{(const S*)links, g.Vb}, Clover<P>{(const S*)clover, g.Vb},
                                              make_geo(g), (float)mu, nrhs, (size_t)g.V * 12, g.V);
   CKL("dslash_blk");
