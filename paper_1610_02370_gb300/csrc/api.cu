@@ -101,6 +101,26 @@ float* field_nrm(const ddtm_field* f, int r) {
   return f->prec == PREC_F16 ? f->nrm.as<float>() + (size_t)r * f->ctx->g.V : nullptr;
 }
 
+ApiFields::ApiFields(ddtm_ctx* c, int prec, int nrhs, int loc) {
+  const size_t V = c->g.V, fb = V * 12 * store2_bytes(prec), nb = prec == PREC_F16 ? V * sizeof(float) : 0;
+  const size_t one = (fb + 255) / 256 * 256 + nb;  // per field and right-hand side
+  batch = 1;
+  if (loc == DDTM_LOC_DEVICE)  // host arrays are staged one right-hand side at a time
+    while (batch < nrhs && batch < 12 && 2 * one * (batch + 1) <= API_KEEP_BYTES) batch++;
+  const size_t da = (fb * batch + 255) / 256 * 256, tot = 2 * (da + (nb * batch + 255) / 256 * 256);
+  char* p;
+  if (tot <= API_KEEP_BYTES) {
+    p = (char*)c->scratch.get("api_fields", tot);
+  } else {
+    own.ensure(tot);
+    p = (char*)own.p;
+  }
+  a = p;
+  b = p + da;
+  an = nb ? (float*)(p + 2 * da) : nullptr;
+  bn = nb ? (float*)(p + 2 * da + (nb * batch + 255) / 256 * 256) : nullptr;
+}
+
 void dslash_field(ddtm_ctx* c, ddtm_field* y, const ddtm_field* x, double mu) {
   ensure_fine_prec(c, x->prec);
   launch_dslash_multi(c->g, x->prec, field_ptr(y, 0), field_nrm(y, 0), field_ptr(x, 0), field_nrm(x, 0),
@@ -305,16 +325,15 @@ int ddtm_apply_D(ddtm_ctx* ctx, double* y, const double* x, int nrhs, double mu,
   if (nrhs == 0) return DDTM_OK;
   ensure_fine_prec(ctx, prec);
   size_t nsp = (size_t)ctx->g.V * 12;
-  ddtm_field fx{ctx, prec, 1}, fy{ctx, prec, 1};
-  field_alloc(&fx);
-  field_alloc(&fy);
-  for (int r = 0; r < nrhs; r++) {
-    const double* din = stage_in(ctx, "canon_in", x + 2 * nsp * r, nsp, loc);
-    double* dout = stage_out(ctx, "canon_out", y + 2 * nsp * r, nsp, loc);
-    launch_spinor_from_canon(ctx->g, prec, fx.data.p, fx.nrm.as<float>(), din, ctx->stream);
-    dslash_field(ctx, &fy, &fx, mu);
-    launch_spinor_to_canon(ctx->g, prec, fy.data.p, fy.nrm.as<float>(), dout, ctx->stream);
-    unstage_out(ctx, y + 2 * nsp * r, dout, nsp, loc);
+  ApiFields f(ctx, prec, nrhs, loc);
+  for (int r = 0; r < nrhs; r += f.batch) {
+    const int R = nrhs - r < f.batch ? nrhs - r : f.batch;
+    const double* din = stage_in(ctx, "canon_in", x + 2 * nsp * r, nsp * R, loc);
+    double* dout = stage_out(ctx, "canon_out", y + 2 * nsp * r, nsp * R, loc);
+    launch_spinor_from_canon(ctx->g, prec, f.a, f.an, din, ctx->stream, R);
+    launch_dslash_multi(ctx->g, prec, f.b, f.bn, f.a, f.an, ctx->links[prec].p, ctx->clover[prec].p, mu, R, ctx->stream);
+    launch_spinor_to_canon(ctx->g, prec, f.b, f.bn, dout, ctx->stream, R);
+    unstage_out(ctx, y + 2 * nsp * r, dout, nsp * R, loc);
   }
   CK(cudaStreamSynchronize(ctx->stream));
   API_END(ctx)
@@ -348,11 +367,15 @@ int ddtm_field_import(ddtm_ctx* ctx, ddtm_field* f, const double* x, int loc) {
   check_loc(loc);
   if (!f || !x || f->ctx != ctx) throw Error(DDTM_ERR_ARG, "invalid arguments");
   size_t nsp = (size_t)ctx->g.V * 12;
+  if (loc == DDTM_LOC_DEVICE) {  // all right-hand sides in one launch
+    launch_spinor_from_canon(ctx->g, f->prec, field_ptr(f, 0), field_nrm(f, 0), x, ctx->stream, f->nrhs);
+    return DDTM_OK;
+  }
   for (int r = 0; r < f->nrhs; r++) {
     const double* din = stage_in(ctx, "canon_in", x + 2 * nsp * r, nsp, loc);
     launch_spinor_from_canon(ctx->g, f->prec, field_ptr(f, r), field_nrm(f, r), din, ctx->stream);
   }
-  if (loc == DDTM_LOC_HOST) CK(cudaStreamSynchronize(ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
   API_END(ctx)
 }
 
@@ -361,6 +384,10 @@ int ddtm_field_export(ddtm_ctx* ctx, const ddtm_field* f, double* x, int loc) {
   check_loc(loc);
   if (!f || !x || f->ctx != ctx) throw Error(DDTM_ERR_ARG, "invalid arguments");
   size_t nsp = (size_t)ctx->g.V * 12;
+  if (loc == DDTM_LOC_DEVICE) {
+    launch_spinor_to_canon(ctx->g, f->prec, field_ptr(f, 0), field_nrm(f, 0), x, ctx->stream, f->nrhs);
+    return DDTM_OK;
+  }
   for (int r = 0; r < f->nrhs; r++) {
     double* dout = stage_out(ctx, "canon_out", x + 2 * nsp * r, nsp, loc);
     launch_spinor_to_canon(ctx->g, f->prec, field_ptr(f, r), field_nrm(f, r), dout, ctx->stream);

@@ -42,9 +42,9 @@ void launch_coarse_even(const CoarseLevel& c, cplx<float>* t, const cplx<float>*
 void launch_parity_copy(const CoarseLevel& c, int parity, cplx<float>* compact, cplx<float>* full, int R, int dir,
                         cudaStream_t st);
 void launch_self_inverse(CoarseLevel& c, double mu_c, cudaStream_t st);
-// canonical FP64 coarse vector <-> column r of an interleaved FP32 batch of R (dir 0: in, 1: out)
+// nr canonical FP64 coarse vectors <-> columns r ... r + nr - 1 of an interleaved FP32 batch of R (dir 0: in, 1: out)
 void launch_coarse_interleave(const CoarseLevel& c, cplx<float>* v, double* canon, int r, int R, int dir,
-                              cudaStream_t st);
+                              cudaStream_t st, int nr = 1);
 
 // coarse_tc.cu: the stencil on tensor cores, FP16 operands and FP32 accumulation.
 // Operands are "images": FP16 copies laid out as the MMA reads them from shared

@@ -205,6 +205,19 @@ struct ddtm_ctx {
 
 namespace ddtm {
 
+// Two internal fields of precision prec for a call on canonical spinors, `batch` right-hand sides at once (as many
+// as fit API_KEEP_BYTES for device arrays, one for host arrays).  Up to API_KEEP_BYTES they are kept with
+// the context's scratch (allocating and freeing them costs 0.1 ms per call, as much as the call itself on a small
+// lattice); larger ones live as long as the object.
+static const size_t API_KEEP_BYTES = (size_t)64 << 20;
+struct ApiFields {
+  int batch;
+  void *a, *b;
+  float *an, *bn;
+  DevBuf own;
+  ApiFields(ddtm_ctx* c, int prec, int nrhs, int loc);
+};
+
 // ---- geometry.cu -------------------------------------------------------------
 void build_geometry(FineGeom& g);
 void build_coarse_geometry(const FineGeom& g, CoarseLevel& c);
@@ -212,9 +225,10 @@ void build_coarse_geometry(const FineGeom& g, CoarseLevel& c);
 void build_coarse_geometry_lat(const int lat[4], CoarseLevel& c);
 // aggregates of b[4] sites on the level-1 lattice of c1
 void build_level1_aggregates(const CoarseLevel& c1, const int b[4], Level1Agg& a);
-// canonical FP64 complex spinor (one rhs) <-> internal field of precision prec
-void launch_spinor_from_canon(const FineGeom& g, int prec, void* d, float* nrm, const double* in, cudaStream_t s);
-void launch_spinor_to_canon(const FineGeom& g, int prec, const void* d, const float* nrm, double* out, cudaStream_t s);
+// R canonical FP64 complex spinors <-> internal fields of precision prec (both at stride 12 V, scales at stride V)
+void launch_spinor_from_canon(const FineGeom& g, int prec, void* d, float* nrm, const double* in, cudaStream_t s, int R = 1);
+void launch_spinor_to_canon(const FineGeom& g, int prec, const void* d, const float* nrm, double* out, cudaStream_t s,
+                            int R = 1);
 // canonical FP64 links -> internal FP64 links
 void launch_links_from_canon(const FineGeom& g, double* out, const double* U, cudaStream_t s);
 // element-wise precision conversion of complex arrays (double2 -> float2 / half2)

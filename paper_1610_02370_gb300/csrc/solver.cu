@@ -909,6 +909,25 @@ static void check_level(ddtm_ctx* c, int level, int lo, int hi_off = 0) {
     throw Error(DDTM_ERR_ARG, "level " + std::to_string(level) + " out of range for a " +
                                   std::to_string(c->p.n_levels) + "-level hierarchy");
 }
+// nrhs canonical coarse vectors -> columns 0 ... nrhs - 1 of an interleaved batch of R, and back: one launch for
+// device arrays, staged one by one for host arrays
+static void coarse_in(ddtm_ctx* c, const CoarseLevel& L, cplx<float>* v, const double* x, int nrhs, int R, int loc) {
+  const size_t nc = (size_t)L.Nc * L.n;
+  const int step = loc == DDTM_LOC_DEVICE ? nrhs : 1;
+  for (int r = 0; r < nrhs; r += step) {
+    const double* din = stage_in(c, "canon_cin", x + 2 * nc * r, nc, loc);
+    launch_coarse_interleave(L, v, const_cast<double*>(din), r, R, 0, c->stream, step);
+  }
+}
+static void coarse_out(ddtm_ctx* c, const CoarseLevel& L, double* x, cplx<float>* v, int nrhs, int R, int loc) {
+  const size_t nc = (size_t)L.Nc * L.n;
+  const int step = loc == DDTM_LOC_DEVICE ? nrhs : 1;
+  for (int r = 0; r < nrhs; r += step) {
+    double* dout = stage_out(c, "canon_cout", x + 2 * nc * r, nc, loc);
+    launch_coarse_interleave(L, v, dout, r, R, 1, c->stream, step);
+    unstage_out(c, x + 2 * nc * r, dout, nc, loc);
+  }
+}
 static CoarseLevel& level_op(ddtm_ctx* c, int level) { return level == 2 ? c->c2 : c->c1; }
 static void check_tc_all(ddtm_ctx* c) {
   check_tc_error(c->c1);
@@ -925,16 +944,15 @@ int ddtm_sap(ddtm_ctx* ctx, double* x, const double* b, int nrhs, double mu, int
   if (nrhs == 0) return DDTM_OK;
   ensure_fine_prec(ctx, prec);
   size_t nsp = (size_t)ctx->g.V * 12;
-  ddtm_field fx{ctx, prec, 1}, fb{ctx, prec, 1};
-  field_alloc(&fx);
-  field_alloc(&fb);
-  for (int r = 0; r < nrhs; r++) {
-    const double* din = stage_in(ctx, "canon_in", b + 2 * nsp * r, nsp, loc);
-    double* dout = stage_out(ctx, "canon_out", x + 2 * nsp * r, nsp, loc);
-    launch_spinor_from_canon(ctx->g, prec, fb.data.p, fb.nrm.as<float>(), din, ctx->stream);
-    sap_run(ctx, prec, fx.data.p, fx.nrm.as<float>(), fb.data.p, fb.nrm.as<float>(), mu, ncycles, nmr, true, 1);
-    launch_spinor_to_canon(ctx->g, prec, fx.data.p, fx.nrm.as<float>(), dout, ctx->stream);
-    unstage_out(ctx, x + 2 * nsp * r, dout, nsp, loc);
+  ApiFields f(ctx, prec, nrhs, loc);
+  for (int r = 0; r < nrhs; r += f.batch) {
+    const int R = nrhs - r < f.batch ? nrhs - r : f.batch;
+    const double* din = stage_in(ctx, "canon_in", b + 2 * nsp * r, nsp * R, loc);
+    double* dout = stage_out(ctx, "canon_out", x + 2 * nsp * r, nsp * R, loc);
+    launch_spinor_from_canon(ctx->g, prec, f.b, f.bn, din, ctx->stream, R);
+    sap_run(ctx, prec, f.a, f.an, f.b, f.bn, mu, ncycles, nmr, true, R);
+    launch_spinor_to_canon(ctx->g, prec, f.a, f.an, dout, ctx->stream, R);
+    unstage_out(ctx, x + 2 * nsp * r, dout, nsp * R, loc);
   }
   CK(cudaStreamSynchronize(ctx->stream));
   API_END(ctx)
@@ -1007,10 +1025,13 @@ int ddtm_set_test_vectors(ddtm_ctx* ctx, int level, const double* v, int nv, int
   size_t nsp = (size_t)ctx->g.V * 12;
   ctx->nv0 = nv;
   ctx->tv0.ensure((size_t)nv * nsp * sizeof(float2));
-  for (int i = 0; i < nv; i++) {
-    const double* din = stage_in(ctx, "canon_in", v + 2 * nsp * i, nsp, loc);
-    launch_spinor_from_canon(ctx->g, PREC_F32, ctx->tv0.as<float2>() + (size_t)i * nsp, nullptr, din, ctx->stream);
-  }
+  if (loc == DDTM_LOC_DEVICE)
+    launch_spinor_from_canon(ctx->g, PREC_F32, ctx->tv0.as<float2>(), nullptr, v, ctx->stream, nv);
+  else
+    for (int i = 0; i < nv; i++) {
+      const double* din = stage_in(ctx, "canon_in", v + 2 * nsp * i, nsp, loc);
+      launch_spinor_from_canon(ctx->g, PREC_F32, ctx->tv0.as<float2>() + (size_t)i * nsp, nullptr, din, ctx->stream);
+    }
   build_hierarchy(ctx);
   if (ctx->p.n_levels == 3 && ctx->a1.tv.p && ctx->a1.nv == ctx->p.nv[1]) build_hierarchy1(ctx);
   CK(cudaStreamSynchronize(ctx->stream));
@@ -1077,16 +1098,15 @@ int ddtm_restrict(ddtm_ctx* ctx, int level, double* cout, const double* x, int n
   cplx<float>* cv = (cplx<float>*)ctx->scratch.get("abi_c32", (size_t)CH * nc * 8);
   for (int r0 = 0; r0 < nrhs; r0 += CH) {
     const int R = nrhs - r0 < CH ? nrhs - r0 : CH;
-    for (int rc = 0; rc < R; rc++) {
-      const double* din = stage_in(ctx, "canon_in", x + 2 * nsp * (r0 + rc), nsp, loc);
-      launch_spinor_from_canon(g, PREC_F32, f + (size_t)rc * nsp, nullptr, din, ctx->stream);
-    }
+    if (loc == DDTM_LOC_DEVICE)
+      launch_spinor_from_canon(g, PREC_F32, f, nullptr, x + 2 * nsp * r0, ctx->stream, R);
+    else
+      for (int rc = 0; rc < R; rc++) {
+        const double* din = stage_in(ctx, "canon_in", x + 2 * nsp * (r0 + rc), nsp, loc);
+        launch_spinor_from_canon(g, PREC_F32, f + (size_t)rc * nsp, nullptr, din, ctx->stream);
+      }
     launch_restrict(g, PREC_F32, cv, f, nullptr, ctx->P0.p, PREC_F32, L.nv, R, R, ctx->stream);
-    for (int rc = 0; rc < R; rc++) {
-      double* dout = stage_out(ctx, "canon_cout", cout + 2 * nc * (r0 + rc), nc, loc);
-      launch_coarse_interleave(L, cv, dout, rc, R, 1, ctx->stream);
-      unstage_out(ctx, cout + 2 * nc * (r0 + rc), dout, nc, loc);
-    }
+    coarse_out(ctx, L, cout + 2 * nc * r0, cv, R, R, loc);
   }
   CK(cudaStreamSynchronize(ctx->stream));
   API_END(ctx)
@@ -1122,11 +1142,12 @@ int ddtm_prolong(ddtm_ctx* ctx, int level, double* x, const double* cin, int nrh
   cplx<float>* cv = (cplx<float>*)ctx->scratch.get("abi_c32", (size_t)CH * nc * 8);
   for (int r0 = 0; r0 < nrhs; r0 += CH) {
     const int R = nrhs - r0 < CH ? nrhs - r0 : CH;
-    for (int rc = 0; rc < R; rc++) {
-      const double* din = stage_in(ctx, "canon_cin", cin + 2 * nc * (r0 + rc), nc, loc);
-      launch_coarse_interleave(L, cv, const_cast<double*>(din), rc, R, 0, ctx->stream);
-    }
+    coarse_in(ctx, L, cv, cin + 2 * nc * r0, R, R, loc);
     launch_prolong(g, PREC_F32, f, nullptr, cv, ctx->P0.p, PREC_F32, L.nv, R, R, 0, ctx->stream);
+    if (loc == DDTM_LOC_DEVICE) {
+      launch_spinor_to_canon(g, PREC_F32, f, nullptr, x + 2 * nsp * r0, ctx->stream, R);
+      continue;
+    }
     for (int rc = 0; rc < R; rc++) {
       double* dout = stage_out(ctx, "canon_out", x + 2 * nsp * (r0 + rc), nsp, loc);
       launch_spinor_to_canon(g, PREC_F32, f + (size_t)rc * nsp, nullptr, dout, ctx->stream);
@@ -1150,18 +1171,11 @@ int ddtm_coarse_solve_batch(ddtm_ctx* ctx, double* x, const double* b, int nrhs,
   cplx<float>* bv = (cplx<float>*)ctx->scratch.get("abi_cb", nc * Rc * 8);
   cplx<float>* xv = (cplx<float>*)ctx->scratch.get("abi_cx", nc * Rc * 8);
   CK(cudaMemsetAsync(bv, 0, nc * Rc * 8, ctx->stream));
-  for (int r = 0; r < nrhs; r++) {
-    const double* din = stage_in(ctx, "canon_cin", b + 2 * nc * r, nc, loc);
-    launch_coarse_interleave(L, bv, const_cast<double*>(din), r, Rc, 0, ctx->stream);
-  }
+  coarse_in(ctx, L, bv, b, nrhs, Rc, loc);
   std::vector<double> rr(Rc, 0.0);
   const int it = coarse_eo_solve(ctx, xv, bv, Rc, mu_c, ctx->p.coarse_restart, ctx->p.coarse_max_restarts,
                                  ctx->p.coarse_tol, rr.data());
-  for (int r = 0; r < nrhs; r++) {
-    double* dout = stage_out(ctx, "canon_cout", x + 2 * nc * r, nc, loc);
-    launch_coarse_interleave(L, xv, dout, r, Rc, 1, ctx->stream);
-    unstage_out(ctx, x + 2 * nc * r, dout, nc, loc);
-  }
+  coarse_out(ctx, L, x, xv, nrhs, Rc, loc);
   CK(cudaStreamSynchronize(ctx->stream));
   check_tc_error(L);
   if (iters) *iters = it;
@@ -1186,10 +1200,7 @@ int ddtm_apply_Dc(ddtm_ctx* ctx, int level, double* y, const double* x, int nrhs
   // all right-hand sides go through one batched stencil pass
   cplx<float>* xv = (cplx<float>*)ctx->scratch.get("abi_c32", nc * nrhs * 8);
   cplx<float>* yv = (cplx<float>*)ctx->scratch.get("abi_c32b", nc * nrhs * 8);
-  for (int r = 0; r < nrhs; r++) {
-    const double* din = stage_in(ctx, "canon_cin", x + 2 * nc * r, nc, loc);
-    launch_coarse_interleave(L, xv, const_cast<double*>(din), r, nrhs, 0, ctx->stream);
-  }
+  coarse_in(ctx, L, xv, x, nrhs, nrhs, loc);
   if (L.prec == PREC_F16) {
     char* xt = (char*)ctx->scratch.get("abi_ct", tc_vector_image_bytes(L, L.Nc, nrhs));
     launch_vector_image(L, xt, xv, 1, L.Nc, nrhs, ctx->stream);
@@ -1208,11 +1219,7 @@ int ddtm_apply_Dc(ddtm_ctx* ctx, int level, double* y, const double* x, int nrhs
   } else {
     launch_coarse_apply_full(L, yv, xv, nrhs, mu, 3, 1.f, 0.f, ctx->stream);
   }
-  for (int r = 0; r < nrhs; r++) {
-    double* dout = stage_out(ctx, "canon_cout", y + 2 * nc * r, nc, loc);
-    launch_coarse_interleave(L, yv, dout, r, nrhs, 1, ctx->stream);
-    unstage_out(ctx, y + 2 * nc * r, dout, nc, loc);
-  }
+  coarse_out(ctx, L, y, yv, nrhs, nrhs, loc);
   CK(cudaStreamSynchronize(ctx->stream));
   check_tc_error(L);
   API_END(ctx)
@@ -1232,16 +1239,9 @@ int ddtm_sap_coarse(ddtm_ctx* ctx, int level, double* x, const double* b, int nr
   cplx<float>* bv = (cplx<float>*)ctx->scratch.get("abi_sapc_b", nc * Rc * 8);
   cplx<float>* xv = (cplx<float>*)ctx->scratch.get("abi_sapc_x", nc * Rc * 8);
   CK(cudaMemsetAsync(bv, 0, nc * Rc * 8, ctx->stream));
-  for (int r = 0; r < nrhs; r++) {
-    const double* din = stage_in(ctx, "canon_cin", b + 2 * nc * r, nc, loc);
-    launch_coarse_interleave(L1, bv, const_cast<double*>(din), r, Rc, 0, ctx->stream);
-  }
+  coarse_in(ctx, L1, bv, b, nrhs, Rc, loc);
   sap_l1(ctx, xv, bv, mu, ncycles, nmr, true, Rc);
-  for (int r = 0; r < nrhs; r++) {
-    double* dout = stage_out(ctx, "canon_cout", x + 2 * nc * r, nc, loc);
-    launch_coarse_interleave(L1, xv, dout, r, Rc, 1, ctx->stream);
-    unstage_out(ctx, x + 2 * nc * r, dout, nc, loc);
-  }
+  coarse_out(ctx, L1, x, xv, nrhs, Rc, loc);
   CK(cudaStreamSynchronize(ctx->stream));
   API_END(ctx)
 }
@@ -1321,16 +1321,22 @@ int ddtm_solve(ddtm_ctx* ctx, double* x, const double* b, int nrhs, double mu, i
     int R = nrhs - r0 < batch ? nrhs - r0 : batch;
     double* bf = (double*)ctx->scratch.get("solve_b", (size_t)R * nsp * 16);
     double* xf = (double*)ctx->scratch.get("solve_x", (size_t)R * nsp * 16);
-    for (int r = 0; r < R; r++) {
-      const double* din = stage_in(ctx, "canon_in", b + 2 * nsp * (r0 + r), nsp, loc);
-      launch_spinor_from_canon(g, PREC_F64, bf + 2 * nsp * r, nullptr, din, ctx->stream);
-    }
+    if (loc == DDTM_LOC_DEVICE)
+      launch_spinor_from_canon(g, PREC_F64, bf, nullptr, b + 2 * nsp * r0, ctx->stream, R);
+    else
+      for (int r = 0; r < R; r++) {
+        const double* din = stage_in(ctx, "canon_in", b + 2 * nsp * (r0 + r), nsp, loc);
+        launch_spinor_from_canon(g, PREC_F64, bf + 2 * nsp * r, nullptr, din, ctx->stream);
+      }
     OuterResult o = outer_fgmres(ctx, xf, bf, mu, R);
-    for (int r = 0; r < R; r++) {
-      double* dout = stage_out(ctx, "canon_out", x + 2 * nsp * (r0 + r), nsp, loc);
-      launch_spinor_to_canon(g, PREC_F64, xf + 2 * nsp * r, nullptr, dout, ctx->stream);
-      unstage_out(ctx, x + 2 * nsp * (r0 + r), dout, nsp, loc);
-    }
+    if (loc == DDTM_LOC_DEVICE)
+      launch_spinor_to_canon(g, PREC_F64, xf, nullptr, x + 2 * nsp * r0, ctx->stream, R);
+    else
+      for (int r = 0; r < R; r++) {
+        double* dout = stage_out(ctx, "canon_out", x + 2 * nsp * (r0 + r), nsp, loc);
+        launch_spinor_to_canon(g, PREC_F64, xf + 2 * nsp * r, nullptr, dout, ctx->stream);
+        unstage_out(ctx, x + 2 * nsp * (r0 + r), dout, nsp, loc);
+      }
     acc.iters = o.iters > acc.iters ? o.iters : acc.iters;
     acc.restarts = o.restarts > acc.restarts ? o.restarts : acc.restarts;
     for (double v : o.relres) acc.max_relres = v > acc.max_relres ? v : acc.max_relres;
