@@ -82,7 +82,9 @@ struct TcPass {
   int nout = 0;
   cplx<float>* y = nullptr;
   const cplx<float>* yin = nullptr;
-  const void* xs = nullptr;  // self vector for the twist, type tag xs_type (1 FP32, 2 FP16)
+  bool y_img = false;        // y is image-ordered FP32 (krylov_tc.h) instead of interleaved
+  const void* xs = nullptr;  // self vector for the twist, type tag xs_type (1 FP32, 2 FP16 interleaved; 3 FP16,
+                             // 4 FP32 in image order)
   int xs_type = 1;
   float sy = 0.f, sres = 1.f, mu_c = 0.f;
   void* yt = nullptr;

@@ -150,7 +150,8 @@ struct TcArgs {
   float2* y;            // y = sy * yin + sres * (acc + i mu_c Gamma5_c xs)   (FP32, optional)
   const float2* yin;
   const void* xs;
-  int xs_half;
+  int xs_type;          // 1 FP32, 2 FP16 interleaved; 3 FP16, 4 FP32 image order
+  int y_img;            // y in image order
   float sy, sres, mu_c;
   char* yt;             // FP16 image of the same result (optional)
   int n, nv, R, r0, Rk; // columns r0 .. r0 + Rk - 1 of R right-hand sides
@@ -330,8 +331,18 @@ __global__ void __launch_bounds__(192, tc_ctas_per_sm(NGJ)) k_coarse_tc(const Tc
           float re = (c ? pa - ob : oa - pb) * a.sres;
           float im = (c ? pb + oa : ob + pa) * a.sres;
           const size_t o = ((size_t)idx * a.n + i) * a.R + r;
+          const size_t oi = (size_t)idx * (a.b_bytes / 2) + img_off(2 * r, i, a.sbo) / 2;  // image order, Im 8 further
           if (a.xs) {
-            const float2 xv = a.xs_half ? ld_f2((const __half2*)a.xs, o) : ld_f2((const float2*)a.xs, o);
+            float2 xv;
+            if (a.xs_type == 3) {
+              const __half* q = (const __half*)a.xs + oi;
+              xv = make_float2(__half2float(q[0]), __half2float(q[8]));
+            } else if (a.xs_type == 4) {
+              const float* q = (const float*)a.xs + oi;
+              xv = make_float2(q[0], q[8]);
+            } else {
+              xv = a.xs_type == 2 ? ld_f2((const __half2*)a.xs, o) : ld_f2((const float2*)a.xs, o);
+            }
             const float m = (i < a.nv ? a.mu_c : -a.mu_c) * a.sres;
             re -= m * xv.y;
             im += m * xv.x;
@@ -341,7 +352,15 @@ __global__ void __launch_bounds__(192, tc_ctas_per_sm(NGJ)) k_coarse_tc(const Tc
             re += a.sy * yv.x;
             im += a.sy * yv.y;
           }
-          if (a.y) a.y[o] = make_float2(re, im);
+          if (a.y) {
+            if (a.y_img) {
+              float* q = reinterpret_cast<float*>(a.y) + oi;
+              q[0] = re;
+              q[8] = im;
+            } else {
+              a.y[o] = make_float2(re, im);
+            }
+          }
           if (img) {
             *reinterpret_cast<__half*>(img + img_off(2 * r, i, a.sbo)) = __float2half_rn(re);
             *reinterpret_cast<__half*>(img + img_off(2 * r + 1, i, a.sbo)) = __float2half_rn(im);
@@ -578,7 +597,7 @@ static void launch_coarse_tc_cps(const CoarseLevel& c, const TcPass& p, int R, c
   bytes += (double)p.nout * t.b_bytes * ((p.self ? 1 : 0) + (p.hops && p.X_hop != p.X_self ? 1 : 0));
   if (p.y) bytes += (double)p.nout * c.n * R * 8;
   if (p.yt) bytes += (double)p.nout * t.b_bytes;
-  if (p.xs) bytes += (double)p.nout * c.n * R * (p.xs_type == 2 ? 4 : 8);
+  if (p.xs) bytes += (double)p.nout * c.n * R * (p.xs_type == 2 || p.xs_type == 3 ? 4 : 8);
   ScopedTimer timer_(p.name, st, R, bytes);
   if (p.nout <= 0) return;
   for (int r0 = 0; r0 < R; r0 += 32) {
@@ -600,8 +619,9 @@ static void launch_coarse_tc_cps(const CoarseLevel& c, const TcPass& p, int R, c
     a.y = reinterpret_cast<float2*>(p.y);
     a.yin = reinterpret_cast<const float2*>(p.yin);
     a.xs = p.xs;
-    if (p.xs && p.xs_type != 1 && p.xs_type != 2) throw Error(DDTM_ERR_ARG, "internal: twist vector type");
-    a.xs_half = p.xs_type == 2;
+    if (p.xs && (p.xs_type < 1 || p.xs_type > 4)) throw Error(DDTM_ERR_ARG, "internal: twist vector type");
+    a.xs_type = p.xs_type;
+    a.y_img = p.y_img ? 1 : 0;
     a.sy = p.sy;
     a.sres = p.sres;
     a.mu_c = p.mu_c;

@@ -14,6 +14,7 @@
 
 #include "blas.h"
 #include "coarse.h"
+#include "krylov_tc.h"
 #include "level1.h"
 #include "common.cuh"
 #include "ddtm_internal.h"
@@ -420,7 +421,131 @@ static int gmres_b(ddtm_ctx* c, const OpF32& A, cplx<float>* x, const cplx<float
   return iters;
 }
 
+// The even-odd GMRES(m) of the tensor-core path (the method and the host's lagging of gmres_b above, one
+// classical Gram-Schmidt pass) on image-ordered vectors: an iteration is the operator's passes and one Arnoldi
+// kernel.  A(w, image, xs, xs_type): w = A v for the FP16 image of v, xs the same v for the twist.
+typedef std::function<void(float*, const void*, const void*, int)> OpImg;
+
+static int gmres_img(ddtm_ctx* c, CoarseLevel& L, const ImgVec& v, int ctas, const OpImg& A, float* x, const float* b, int m,
+                     int max_restarts, double tol, double* relres, const std::string& op_key) {
+  const int R = v.t.R;
+  const size_t ne = v.entries(), vb = ne * sizeof(__half);
+  char* V = (char*)c->scratch.get("cgi_V", (size_t)(m + 1) * vb);
+  float* w = (float*)c->scratch.get("cgi_w", ne * sizeof(float));
+  char* xh = (char*)c->scratch.get("cgi_xh", vb);
+  auto Vj = [&](int j) { return (void*)(V + (size_t)j * vb); };
+  GsBuffers gb;
+  const size_t nH = (size_t)R * (m + 1) * m, ncs = (size_t)R * m, ng = (size_t)R * (m + 1), nh = (size_t)(m + 1) * R;
+  double2* st2 = (double2*)c->scratch.get("cgi_state", (nH + 2 * ncs + ng + 2 * nh) * sizeof(double2) + 2 * (size_t)R * sizeof(double));
+  ArnoldiDev ad;
+  ad.H = st2;
+  ad.cs = ad.H + nH;
+  ad.sn = ad.cs + ncs;
+  ad.g = ad.sn + ncs;
+  gb.h = ad.g + ng;
+  double2* y = gb.h + nh;
+  ad.scale = nullptr;
+  ad.bn = (double*)(y + nh);
+  ad.est = ad.bn + R;
+  ad.m = m;
+  ad.R = R;
+  char* pb = (char*)c->scratch.get("cgi_part", (size_t)m * R * ctas * sizeof(float2) + (size_t)R * ctas * sizeof(double) + 64);
+  gb.part = (float2*)pb;
+  gb.npart = (double*)(gb.part + (size_t)m * R * ctas);
+  gb.bar = (unsigned*)(gb.npart + (size_t)R * ctas);
+  gb.err = L.tc_err.as<int>();
+  double* est_h = (double*)c->scratch_host("cgi_est", 2 * (size_t)R * sizeof(double));
+  cudaEvent_t ev[2];
+  c->events("cgi", ev);
+  CK(cudaMemsetAsync(x, 0, ne * sizeof(float), c->stream));
+  CK(cudaMemsetAsync(w, 0, ne * sizeof(float), c->stream));  // its padding entries stay zero
+  CK(cudaMemsetAsync(gb.bar, 0, 3 * sizeof(unsigned), c->stream));
+  std::vector<double> est(R, 0.0);
+  // the estimates of slot, once their kernel has run; true when every system has converged
+  auto converged = [&](int slot) {
+    CK(cudaEventSynchronize(ev[slot]));
+    bool done = true;
+    for (int r = 0; r < R; r++) {
+      est[r] = est_h[(size_t)slot * R + r];
+      if (!std::isfinite(est[r])) throw Error(DDTM_ERR_NAN, "non-finite residual in the coarse GMRES");
+      done = done && est[r] <= tol;
+    }
+    return done;
+  };
+  int iters = 0;
+  bool done = false;
+  cudaStream_t st = c->stream;  // follows c->stream into a capture
+  for (int cyc = 0; cyc <= max_restarts && !done; cyc++) {
+    if (cyc == 0) {
+      CK(cudaMemcpyAsync(w, b, ne * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
+    } else {
+      launch_img_half(v, xh, x, c->stream);
+      A(w, xh, x, 4);
+      launch_img_residual(v, w, b, c->stream);
+    }
+    launch_gs_step(v, V, vb, 0, w, Vj(0), ad, cyc == 0, est_h + R, gb, c->stream);
+    CK(cudaEventRecord(ev[1], c->stream));
+    int k = 0;
+    for (int j = 0; j < m; j++) {
+      auto iteration = [&]() {
+        A(w, Vj(j), Vj(j), 3);
+        launch_gs_step(v, V, vb, j + 1, w, j < m - 1 ? Vj(j + 1) : nullptr, ad, 0, est_h + (size_t)(j & 1) * R, gb, c->stream);
+      };
+      char kb[160];
+      snprintf(kb, sizeof(kb), "cgi|j%d|R%d|m%d|s%d|G%d|est%p|", j, R, m, v.nsites, ctas, (void*)est_h);
+      run_as_graph(c, std::string(kb) + op_key, &st, iteration);
+      CK(cudaEventRecord(ev[j & 1], c->stream));
+      k = j + 1;
+      iters++;
+      if (converged((j + 1) & 1)) {  // the start's estimates, or the previous iteration's: iteration j is discarded
+        k = j;
+        iters--;
+        done = true;
+        break;
+      }
+    }
+    if (!done) done = converged((k - 1) & 1);
+    launch_arnoldi_solve(ad, k, y, c->stream);
+    launch_img_combine(v, x, V, vb, k, y, c->stream);
+  }
+  for (int r = 0; r < R; r++) relres[r] = est[r];
+  return iters;
+}
+
 // ---- coarsest level: even-odd GMRES (Sec. 2.5) ------------------------------------------
+// The two tensor-core passes of D_hat = D_oo - D_oe D_ee^-1 D_eo on an odd-site image:
+// tt = -D_ee^-1 D_eo in, from the products D_ee^-1(e) A_d(e) (one pass, no intermediate), and
+// out = (D_oo + i mu_c Gamma5_c) in + D_oe tt (y and the twist's vector set by the caller)
+static TcPass hop_even_pass(const CoarseLevel& L, const void* img, void* tt) {
+  TcPass h;
+  h.name = "coarse_tc_hop_even";
+  h.hops = true;
+  h.A_hop = L.Dhopt.p;
+  h.hop_by_slot = true;
+  h.X_hop = img;
+  h.tab = L.nbr_eo.as<int>();
+  h.osite = L.even.as<int>();
+  h.nout = (int)L.h_even.size();
+  h.sres = -1.f;
+  h.yt = tt;
+  return h;
+}
+static TcPass odd_pass(const CoarseLevel& L, const void* img, const void* tt, double mu_c) {
+  TcPass o;
+  o.name = "coarse_tc_odd";
+  o.self = o.hops = true;
+  o.A_self = L.Dct.p;
+  o.a_self_stride = 9 * (size_t)tc_geom(L.n, 1).a_bytes;
+  o.self_by_site = true;
+  o.A_hop = L.Dct.p;
+  o.X_self = img;
+  o.X_hop = tt;
+  o.tab = L.nbr_oe.as<int>();
+  o.osite = L.odd.as<int>();
+  o.nout = (int)L.h_odd.size();
+  o.mu_c = (float)mu_c;
+  return o;
+}
 // D_c(mu_c) phi = eta for a batch of Rc interleaved coarse vectors:
 // rhat = eta_o - D_oe D_ee^-1 eta_e;  GMRES on D_hat = D_oo - D_oe D_ee^-1 D_eo;
 // phi_e = D_ee^-1 (eta_e - D_eo phi_o).  Returns the iteration count; relres
@@ -440,6 +565,34 @@ int coarse_eo_solve(ddtm_ctx* c, cplx<float>* x_full, const cplx<float>* b_full,
   launch_parity_copy(L, 1, bo, (cplx<float>*)b_full, Rc, 0, c->stream);
   launch_coarse_even(L, te, be, nullptr, Rc, 1.f, 0.f, c->stream);                 // te = D_ee^-1 eta_e
   launch_coarse_apply_odd(L, bo, nullptr, te, Rc, mu_c, 2, -1.f, 1.f, c->stream);   // rhat = eta_o - D_oe te
+  char ok[96];  // what the operator's launch arguments depend on besides buffers
+  snprintf(ok, sizeof(ok), "eo|mu%.17g|p%d|lev%p", mu_c, L.prec, (const void*)&L);
+  const ImgVec v{tc_geom(L.n, Rc), (int)no};
+  const int ctas = L.prec == PREC_F16 && tol >= 1e-3 ? gs_ctas(v, restart) : 0;
+  if (ctas > 0) {
+    // tensor cores on image-ordered vectors; tighter tolerances need the second Gram-Schmidt pass of gmres_b
+    char* tt = (char*)c->scratch.get("ceo_tt", tc_vector_image_bytes(L, (int)ne, Rc));
+    float* bi = (float*)c->scratch.get("ceo_bi", v.entries() * sizeof(float));
+    float* xi = (float*)c->scratch.get("ceo_xi", v.entries() * sizeof(float));
+    launch_img_order(v, bi, bo, 0, c->stream);
+    OpImg Dimg = [&, tt](float* out, const void* img, const void* xs, int xs_type) {
+      TcPass h = hop_even_pass(L, img, tt);
+      launch_coarse_tc(L, h, Rc, c->stream);
+      TcPass o = odd_pass(L, img, tt, mu_c);
+      o.y = reinterpret_cast<cplx<float>*>(out);
+      o.y_img = true;
+      o.xs = xs;
+      o.xs_type = xs_type;
+      launch_coarse_tc(L, o, Rc, c->stream);
+    };
+    const int it = gmres_img(c, L, v, ctas, Dimg, xi, bi, restart, max_restarts, tol, relres, std::string(ok));
+    launch_img_order(v, xi, xo, 1, c->stream);
+    launch_coarse_even(L, te, be, xo, Rc, 1.f, -1.f, c->stream);  // phi_e = D_ee^-1 (eta_e - D_eo phi_o)
+    launch_parity_copy(L, 0, te, x_full, Rc, 1, c->stream);
+    launch_parity_copy(L, 1, xo, x_full, Rc, 1, c->stream);
+    c->coarse_iters += (long)it * Rc;
+    return it;
+  }
   OpF32 Dhat;
   if (L.prec == PREC_F16) {
     // tensor cores: FP16 images of the operand vectors, FP32 accumulation;
@@ -447,37 +600,13 @@ int coarse_eo_solve(ddtm_ctx* c, cplx<float>* x_full, const cplx<float>* b_full,
     const size_t img_o = tc_vector_image_bytes(L, (int)no, Rc), img_e = tc_vector_image_bytes(L, (int)ne, Rc);
     char* vt = (char*)c->scratch.get("ceo_vt", img_o);
     char* tt = (char*)c->scratch.get("ceo_tt", img_e);
-    const size_t ab = tc_geom(L.n, 1).a_bytes;
-    Dhat = [&, vt, tt, ab](cplx<float>* out, const void* in, int in_type) {
+    Dhat = [&, vt, tt](cplx<float>* out, const void* in, int in_type) {
       launch_vector_image(L, vt, in, in_type, (int)no, Rc, c->stream);
-      TcPass h;  // tt = -D_ee^-1 D_eo in, from the products D_ee^-1(e) A_d(e) (one pass, no intermediate)
-      h.name = "coarse_tc_hop_even";
-      h.hops = true;
-      h.A_hop = L.Dhopt.p;
-      h.hop_by_slot = true;
-      h.X_hop = vt;
-      h.tab = L.nbr_eo.as<int>();
-      h.osite = L.even.as<int>();
-      h.nout = (int)ne;
-      h.sres = -1.f;
-      h.yt = tt;
-      launch_coarse_tc(L, h, Rc, c->stream);
-      TcPass o;  // out = (D_oo + i mu_c Gamma5_c) in + D_oe tt
-      o.name = "coarse_tc_odd";
-      o.self = o.hops = true;
-      o.A_self = L.Dct.p;
-      o.a_self_stride = 9 * ab;
-      o.self_by_site = true;
-      o.A_hop = L.Dct.p;
-      o.X_self = vt;
-      o.X_hop = tt;
-      o.tab = L.nbr_oe.as<int>();
-      o.osite = L.odd.as<int>();
-      o.nout = (int)no;
+      launch_coarse_tc(L, hop_even_pass(L, vt, tt), Rc, c->stream);
+      TcPass o = odd_pass(L, vt, tt, mu_c);
       o.y = out;
       o.xs = in;
       o.xs_type = in_type;
-      o.mu_c = (float)mu_c;
       launch_coarse_tc(L, o, Rc, c->stream);
     };
   } else {
@@ -489,8 +618,6 @@ int coarse_eo_solve(ddtm_ctx* c, cplx<float>* x_full, const cplx<float>* b_full,
     };
   }
   // FP16 Krylov basis with the tensor-core stencil (which reads FP16 operands anyway)
-  char ok[96];  // what the operator's launch arguments depend on besides buffers
-  snprintf(ok, sizeof(ok), "eo|mu%.17g|p%d|lev%p", mu_c, L.prec, (const void*)&L);
   int it = gmres_b(c, Dhat, xo, bo, no * n, Rc, restart, max_restarts, tol, relres, "cgm", L.prec == PREC_F16,
                    std::string(ok));
   launch_coarse_even(L, te, be, xo, Rc, 1.f, -1.f, c->stream);  // phi_e = D_ee^-1 (eta_e - D_eo phi_o)
