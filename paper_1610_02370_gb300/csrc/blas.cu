@@ -471,10 +471,16 @@ __global__ void k_bscale(const double2* __restrict__ a, const TX* x, TY* y, size
   }
 }
 
+// grid.y = right-hand side (fields at stride 12 V, FP16 scales at stride V)
 template <int PI, int PO>
 __global__ void k_field_convert(Spinor<PO> out, Spinor<PI> in, long V) {
   long s = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= V) return;
+  const size_t r = blockIdx.y;
+  in.d += r * 12 * V;
+  out.d += r * 12 * V;
+  if (Prec<PI>::scaled) in.nrm += r * V;
+  if (Prec<PO>::scaled) out.nrm += r * V;
   int blk = (int)(s / in.Vb), loc = (int)(s - (long)blk * in.Vb);
   cplx<typename Prec<PI>::real> a[12];
   in.loadw(blk, loc, a);
@@ -482,6 +488,44 @@ __global__ void k_field_convert(Spinor<PO> out, Spinor<PI> in, long V) {
 #pragma unroll
   for (int c = 0; c < 12; c++) b[c] = cplx<typename Prec<PO>::real>(a[c].re, a[c].im);
   out.store(blk, loc, b);
+}
+
+// FP32 -> FP64, exactly, by integer operations: the conversion instruction shares the FP64 pipe, which is the bound
+// of the kernel below
+__device__ __forceinline__ double f2d(float f) {
+  const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+  if (e == 0 || e == 0x7f800000u) return (double)f;  // zero, subnormal, infinity, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double f2d(double f) { return f; }
+
+// x_r += sum_j y[j R + r] Z_j,r in FP64, Z_j the stored fields of step j at stride jstride (scales at stride jnstride):
+// x is read and written once, Z read in its storage precision (the FP64 copy of each Z_j and one update per j
+// moved 13 times as much).  Bound by FP64 arithmetic.
+template <int P>
+__global__ void __launch_bounds__(256) k_fine_update(double2* __restrict__ x, const typename Prec<P>::store2* __restrict__ Z,
+                                                     const float* __restrict__ Zn, size_t jstride, size_t jnstride, int nj,
+                                                     const double2* __restrict__ y, int R, int Vb, long V) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* yc = reinterpret_cast<double2*>(smem_raw);  // [nj]
+  const size_t r = blockIdx.y;
+  for (int j = threadIdx.x; j < nj; j += blockDim.x) yc[j] = y[(size_t)j * R + r];
+  __syncthreads();
+  const size_t n = (size_t)12 * V, i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // one component of one site
+  if (i >= n) return;
+  const size_t site = i / (12 * (size_t)Vb) * Vb + i % Vb;  // of entry [blk][component][loc]
+  double2 acc = x[r * n + i];
+#pragma unroll 4
+  for (int j = 0; j < nj; j++) {
+    const cplx<typename Prec<P>::real> f = ldw(Z + (size_t)j * jstride + r * n + i);
+    typename Prec<P>::real s = 1;
+    if (Prec<P>::scaled) s = Zn[(size_t)j * jnstride + r * V + site];
+    const double zr = f2d(s * f.re), zi = f2d(s * f.im);
+    const double2 c = yc[j];
+    acc.x = fma(c.x, zr, fma(-c.y, zi, acc.x));
+    acc.y = fma(c.x, zi, fma(c.y, zr, acc.y));
+  }
+  x[r * n + i] = acc;
 }
 
 // ---- host side -------------------------------------------------------------------------
@@ -965,9 +1009,15 @@ void launch_arnoldi_solve(const ArnoldiDev& a, int k, double2* y, cudaStream_t s
 }
 
 void launch_field_convert(const FineGeom& g, int pin, const void* in, const float* inn, int pout, void* out, float* outn,
-                          cudaStream_t st) {
-  ScopedTimer timer_("field_convert", st);
-  unsigned grid = (unsigned)((g.V + 127) / 128);
+                          cudaStream_t st, int R) {
+  ScopedTimer timer_("field_convert", st, R);
+  if (pin == pout) {
+    CK(cudaMemcpyAsync(out, in, (size_t)R * g.V * 12 * (pin == PREC_F64 ? 16 : pin == PREC_F32 ? 8 : 4),
+                       cudaMemcpyDeviceToDevice, st));
+    if (pin == PREC_F16) CK(cudaMemcpyAsync(outn, inn, (size_t)R * g.V * 4, cudaMemcpyDeviceToDevice, st));
+    return;
+  }
+  const dim3 grid((unsigned)((g.V + 127) / 128), R);
 #define CONV(A, B, SA, SB)                                                                          \
   k_field_convert<A, B><<<grid, 128, 0, st>>>(Spinor<B>{(SB*)out, outn, g.Vb}, Spinor<A>{(SA*)in, (float*)inn, g.Vb}, g.V)
   if (pin == PREC_F64 && pout == PREC_F32) CONV(PREC_F64, PREC_F32, double2, float2);
@@ -975,14 +1025,26 @@ void launch_field_convert(const FineGeom& g, int pin, const void* in, const floa
   else if (pin == PREC_F32 && pout == PREC_F64) CONV(PREC_F32, PREC_F64, float2, double2);
   else if (pin == PREC_F32 && pout == PREC_F16) CONV(PREC_F32, PREC_F16, float2, __half2);
   else if (pin == PREC_F16 && pout == PREC_F64) CONV(PREC_F16, PREC_F64, __half2, double2);
-  else if (pin == PREC_F16 && pout == PREC_F32) CONV(PREC_F16, PREC_F32, __half2, float2);
-  else if (pin == pout) {
-    CK(cudaMemcpyAsync(out, in, (size_t)g.V * 12 * (pin == PREC_F64 ? 16 : pin == PREC_F32 ? 8 : 4),
-                       cudaMemcpyDeviceToDevice, st));
-    if (pin == PREC_F16) CK(cudaMemcpyAsync(outn, inn, (size_t)g.V * 4, cudaMemcpyDeviceToDevice, st));
-  }
+  else CONV(PREC_F16, PREC_F32, __half2, float2);
 #undef CONV
   CKL("field_convert");
+}
+
+template <int P>
+static void fine_update_t(const FineGeom& g, double* x, const void* Z, const float* Zn, int nj, const double2* y, int R,
+                          cudaStream_t st) {
+  const size_t n = (size_t)12 * g.V, smem = (size_t)nj * sizeof(double2);
+  k_fine_update<P><<<dim3((unsigned)((n + 255) / 256), R), 256, smem, st>>>(
+      (double2*)x, (const typename Prec<P>::store2*)Z, Zn, (size_t)R * n, (size_t)R * g.V, nj, y, R, g.Vb, g.V);
+}
+void launch_fine_update(const FineGeom& g, double* x, int prec, const void* Z, const float* Zn, int nj, const double2* y,
+                        int R, cudaStream_t st) {
+  ScopedTimer timer_("fine_update", st, R, (double)R * g.V * 12 * (32.0 + nj * (prec == PREC_F64 ? 16 : prec == PREC_F32 ? 8 : 4)));
+  if (nj <= 0) return;
+  if (prec == PREC_F64) fine_update_t<PREC_F64>(g, x, Z, Zn, nj, y, R, st);
+  else if (prec == PREC_F32) fine_update_t<PREC_F32>(g, x, Z, Zn, nj, y, R, st);
+  else fine_update_t<PREC_F16>(g, x, Z, Zn, nj, y, R, st);
+  CKL("fine_update");
 }
 
 }  // namespace ddtm

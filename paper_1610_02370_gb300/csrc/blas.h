@@ -78,7 +78,11 @@ void launch_arnoldi_step(const ArnoldiDev& a, int j, const double2* h, const dou
 // y[i*R + r] from the triangular systems of the first k columns
 void launch_arnoldi_solve(const ArnoldiDev& a, int k, double2* y, cudaStream_t st);
 
+// R fields at stride 12 V (FP16 scales at stride V)
 void launch_field_convert(const FineGeom& g, int pin, const void* in, const float* inn, int pout, void* out, float* outn,
-                          cudaStream_t st);
+                          cudaStream_t st, int R = 1);
+// x_r += sum_{j < nj} y[j R + r] Z_j,r in FP64 for R fine fields; Z_j of precision prec at stride 12 V R (scales V R)
+void launch_fine_update(const FineGeom& g, double* x, int prec, const void* Z, const float* Zn, int nj, const double2* y,
+                        int R, cudaStream_t st);
 
 }  // namespace ddtm

@@ -842,18 +842,14 @@ OuterResult outer_fgmres(ddtm_ctx* c, double* x, const double* b, double mu, int
       const void* vin = Vj(j);
       const float* vinn = nullptr;
       if (sp != cp) {
-        for (int r = 0; r < R; r++)
-          launch_field_convert(g, cp, (char*)Vj(j) + (size_t)r * cb, nullptr, sp, vsb + (size_t)r * fb,
-                               sp == PREC_F16 ? vsn + (size_t)r * g.V : nullptr, c->stream);
+        launch_field_convert(g, cp, Vj(j), nullptr, sp, vsb, sp == PREC_F16 ? vsn : nullptr, c->stream, R);
         vin = vsb;
         vinn = sp == PREC_F16 ? vsn : nullptr;
       }
       mg_precondition(c, sp, Zj(j), Zjn(j), vin, vinn, mu, R);
       const void* zin = Zj(j);
       if (sp != cp) {
-        for (int r = 0; r < R; r++)
-          launch_field_convert(g, sp, (char*)Zj(j) + (size_t)r * fb, sp == PREC_F16 ? Zjn(j) + (size_t)r * g.V : nullptr,
-                               cp, t32 + (size_t)r * cb, nullptr, c->stream);
+        launch_field_convert(g, sp, Zj(j), Zjn(j), cp, t32, nullptr, c->stream, R);
         zin = t32;
       }
       Dcyc(w, zin);
@@ -879,18 +875,7 @@ OuterResult outer_fgmres(ddtm_ctx* c, double* x, const double* b, double mu, int
     }
     if (!cyc_done) CK(cudaEventSynchronize(ev[(k - 1) & 1]));
     launch_arnoldi_solve(ad, k, y, c->stream);
-    // x += sum_j y_j Z_j in FP64
-    double* t64 = (double*)c->scratch.get("out_t64", (size_t)R * n * 16);
-    for (int j = 0; j < k; j++) {
-      const double* zj = (const double*)Zj(j);
-      if (sp != PREC_F64) {
-        for (int r = 0; r < R; r++)
-          launch_field_convert(g, sp, (char*)Zj(j) + (size_t)r * fb, sp == PREC_F16 ? Zjn(j) + (size_t)r * g.V : nullptr,
-                               PREC_F64, t64 + 2 * (size_t)r * n, nullptr, c->stream);
-        zj = t64;
-      }
-      B.maxpy_dev(s64(x), s64(zj), 0, 1, y + (size_t)j * R, +1.0, nullptr);
-    }
+    launch_fine_update(g, x, sp, Z, sp == PREC_F16 ? Zn : nullptr, k, y, R, c->stream);  // x += sum_j y_j Z_j in FP64
   }
   return res;
 }
@@ -935,14 +920,10 @@ void run_setup(ddtm_ctx* c, double mu, uint64_t seed, bool update = false, int n
   char* xs = (char*)c->scratch.get("setup_x", (size_t)nv * fb);
   float* xsn = (float*)c->scratch.get("setup_xn", (size_t)nv * g.V * 4);
   auto to_sp = [&]() {
-    for (int i = 0; i < nv; i++)
-      launch_field_convert(g, PREC_F32, tv + (size_t)i * n, nullptr, sp, bs + (size_t)i * fb,
-                           sp == PREC_F16 ? bsn + (size_t)i * g.V : nullptr, c->stream);
+    launch_field_convert(g, PREC_F32, tv, nullptr, sp, bs, sp == PREC_F16 ? bsn : nullptr, c->stream, nv);
   };
   auto from_sp = [&]() {
-    for (int i = 0; i < nv; i++)
-      launch_field_convert(g, sp, xs + (size_t)i * fb, sp == PREC_F16 ? xsn + (size_t)i * g.V : nullptr, PREC_F32,
-                           tv + (size_t)i * n, nullptr, c->stream);
+    launch_field_convert(g, sp, xs, sp == PREC_F16 ? xsn : nullptr, PREC_F32, tv, nullptr, c->stream, nv);
   };
   float* bnp = sp == PREC_F16 ? bsn : nullptr;
   float* xnp = sp == PREC_F16 ? xsn : nullptr;
