@@ -269,6 +269,223 @@ __global__ void __launch_bounds__(256, 1) k_galerkin_rows(float2* __restrict__ D
   }
 }
 
+// ---- Galerkin build with matrix instructions -----------------------------------------
+// The same products, for FP16 coarse storage: one CTA per (aggregate A, row chirality s) keeps the nv rows of P on A
+// as FP16 in shared memory and forms, for each part d (self, then the faces) and X sites at a time, the
+// chirality-s components y of all n columns in FP32; their projections are a dense contraction
+//   D[i][j] = sum over (component, site) conj(P_i) y_j
+// done by mma.sync m16n8k8 in TF32: P's FP16 entries are exact in TF32, y goes in as hi + lo (21 bits) and sums are
+// FP32, so the result is as exact as the FP32 sums of k_galerkin_rows it replaces.  (The operands sit in registers and shared memory
+// where the FP32 stencil leaves them; the contraction is 43 GFLOP at 16^3 x 32, a small part of the time, so the
+// tensor-memory path would not pay for staging operand images.)  16^3 x 32, n = 48: 2.72 ms, k_galerkin_rows<2> 6.95 ms
+// (its projections took 17 shared-memory loads per 32 multiply-adds and a warp reduction per entry); what is left is
+// the latency of the P and link loads at 12 warps per SM.  Columns are spread over the threads X sites x
+// (GM_THREADS / X) column groups, GM_CPT columns per thread sharing each link.
+static const int GM_THREADS = 384, GM_CPT = 4;
+
+__device__ __forceinline__ uint32_t to_tf32(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ void mma_tf32(float c[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// acc[cc] += chirality-s part of the hop (MU, FWD) of GM_CPT columns col0 + cc cstep read at (blk, loc) of P
+// (columns beyond n repeat the last one; they are not stored)
+template <int MU, bool FWD>
+__device__ __forceinline__ void galerkin_hop(cplx<float> (&acc)[GM_CPT][6], const float2* __restrict__ P, const Links<PREC_F32>& U,
+                                             float sign, int s, int A, int own, int blk, int loc, int nv, int Vb, int n,
+                                             int col0, int cstep) {
+  cplx<float> u[9];
+  if (FWD) U.load(A, own, MU, u);
+  else U.load(blk, loc, MU, u);
+#pragma unroll
+  for (int cc = 0; cc < GM_CPT; cc++) {
+    const int col = col0 + cc * cstep < n ? col0 + cc * cstep : n - 1;
+    const int sp = col >= nv ? 1 : 0, j = col - sp * nv;
+    cplx<float> v[6], h[6], w[6];
+    const float2* src = P + pix(blk, sp, j, 0, loc, nv, Vb);
+#pragma unroll
+    for (int c = 0; c < 6; c++) v[c] = ld(src + (size_t)c * Vb);
+    // upper half of the projection: sp = 0 the column itself, sp = 1 -G l (forward), +G l (backward)
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      cplx<float> g0, g1;
+      apply_G<float>(MU, v[c], v[3 + c], g0, g1);
+      h[c] = sp ? (FWD ? -g0 : g0) : v[c];
+      h[3 + c] = sp ? (FWD ? -g1 : g1) : v[3 + c];
+    }
+    if (FWD) mul_U<float>(u, h, w);
+    else mul_Udag<float>(u, h, w);
+    // s = 0: w; s = 1: mu = 0 forward -w, backward w; mu = k forward G w, backward -G w
+    const float q = s ? (((MU == 0) == FWD) ? -sign : sign) : sign;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      cplx<float> g0, g1;
+      apply_G<float>(MU, w[c], w[3 + c], g0, g1);
+      const cplx<float> o0 = s ? g0 : w[c], o1 = s ? g1 : w[3 + c];
+      acc[cc][c].re = fmaf(q, o0.re, acc[cc][c].re);
+      acc[cc][c].im = fmaf(q, o0.im, acc[cc][c].im);
+      acc[cc][3 + c].re = fmaf(q, o1.re, acc[cc][3 + c].re);
+      acc[cc][3 + c].im = fmaf(q, o1.im, acc[cc][3 + c].im);
+    }
+  }
+}
+
+// acc[cc] += site term (chirality s, packed at cp) of the columns of that chirality
+__device__ __forceinline__ void galerkin_site(cplx<float> (&acc)[GM_CPT][6], const float2* __restrict__ P,
+                                              const float2* __restrict__ cp, int s, int A, int loc, int nv, int Vb, int n,
+                                              int col0, int cstep) {
+  cplx<float> t[18];
+#pragma unroll
+  for (int q = 0; q < 18; q++) t[q] = ld(cp + (size_t)q * Vb);
+#pragma unroll
+  for (int cc = 0; cc < GM_CPT; cc++) {
+    const int col = col0 + cc * cstep;
+    if (col < n && (col >= nv) == (s == 1)) {
+      cplx<float> v[6];
+#pragma unroll
+      for (int c = 0; c < 6; c++) v[c] = ld(P + pix(A, s, col - s * nv, c, loc, nv, Vb));
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        acc[cc][2 * q] = acc[cc][2 * q] + t[q].re * v[2 * q];
+        acc[cc][2 * q + 1] = acc[cc][2 * q + 1] + t[q].im * v[2 * q + 1];
+      }
+#pragma unroll
+      for (int i = 0; i < 5; i++)
+#pragma unroll
+        for (int j = 1; j < 6; j++)
+          if (j > i) {
+            const int slot = 3 + i * 5 - i * (i - 1) / 2 + (j - i - 1);
+            cmac(acc[cc][i], t[slot], v[j]);
+            cmac_conj(acc[cc][j], t[slot], v[i]);
+          }
+    }
+  }
+}
+
+// one 16 x 8 tile of the projections of a chunk of X sites
+template <int X>
+__device__ __forceinline__ void galerkin_tile(float (&cr)[4], float (&ci)[4], const __half2* __restrict__ Ps, const float2* __restrict__ Bs,
+                                              const int* sites, int tile, int ntile, int nv, int rs, int Vb, int lane) {
+  constexpr int BS = 6 * X + 4;
+  const int n = 2 * nv, mt = tile / ntile, nt = tile - mt * ntile, t = lane & 3, gr = lane >> 2;
+  const int i0 = mt * 16 + gr < nv ? mt * 16 + gr : nv - 1, i1 = mt * 16 + gr + 8 < nv ? mt * 16 + gr + 8 : nv - 1;
+  const int col = nt * 8 + gr < n ? nt * 8 + gr : n - 1;  // rows and columns beyond the edge are not stored
+  const __half2 *pa = Ps + (size_t)i0 * rs, *pb = Ps + (size_t)i1 * rs;
+  const float2* pc = Bs + (size_t)col * BS;
+#pragma unroll 1
+  for (int c = 0; c < 6; c++)
+#pragma unroll
+    for (int x0 = 0; x0 < X; x0 += 4) {
+      const int st = c * Vb + sites[x0 + t];
+      const float2 a = __half22float2(pa[st]), b = __half22float2(pb[st]), y = pc[c * X + x0 + t];
+      const uint32_t ar = __float_as_uint(a.x), ai = __float_as_uint(a.y), br = __float_as_uint(b.x), bi = __float_as_uint(b.y),
+                     an = __float_as_uint(-a.y), bn = __float_as_uint(-b.y);
+      const uint32_t hr = to_tf32(y.x), hi = to_tf32(y.y);
+      const uint32_t lr = to_tf32(y.x - __uint_as_float(hr)), li = to_tf32(y.y - __uint_as_float(hi));
+      mma_tf32(cr, ar, br, ai, bi, hr, hi);
+      mma_tf32(ci, an, bn, ar, br, hr, hi);
+      mma_tf32(cr, ar, br, ai, bi, lr, li);
+      mma_tf32(ci, an, bn, ar, br, lr, li);
+    }
+}
+
+template <int X>
+__global__ void __launch_bounds__(GM_THREADS, 1) k_galerkin_mma(float2* __restrict__ Dc, const float2* __restrict__ P,
+                                                                Links<PREC_F32> U, Clover<PREC_F32> C, Geo g, FaceTables f,
+                                                                int nv, int rs) {
+  constexpr int BS = 6 * X + 4;    // entries per column of y
+  constexpr int CG = GM_THREADS / X;  // column groups
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int sites[X];
+  const int Vb = g.Vb, A = blockIdx.x >> 1, s = blockIdx.x & 1, n = 2 * nv;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __half2* Ps = reinterpret_cast<__half2*>(smem_raw);                       // [nv][rs], entry comp * Vb + site
+  float2* Bs = reinterpret_cast<float2*>(smem_raw + (size_t)nv * rs * 4);   // [n][BS], entry comp * X + x
+  for (int e = threadIdx.x; e < nv * 6 * Vb; e += GM_THREADS) {
+    const int i = e / (6 * Vb), q = e - i * 6 * Vb;
+    Ps[(size_t)i * rs + q] = __float22half2_rn(__ldg(P + pix(A, s, i, 0, 0, nv, Vb) + q));
+  }
+  const int x = threadIdx.x % X, cg = threadIdx.x / X;
+  const int ntile = (n + 7) / 8, tiles = (nv + 15) / 16 * ntile;  // 16 x 8 tiles, at most two per warp
+  for (int d = 0; d < 9; d++) {
+    const int nsite = d ? f.off[d] - f.off[d - 1] : Vb;
+    float cr0[4] = {0.f, 0.f, 0.f, 0.f}, ci0[4] = {0.f, 0.f, 0.f, 0.f}, cr1[4] = {0.f, 0.f, 0.f, 0.f}, ci1[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int c0 = 0; c0 < nsite; c0 += X) {
+      // ---- y of X sites, all columns
+      const bool in = c0 + x < nsite;
+      const int loc = !in ? 0 : d ? f.list[f.off[d - 1] + c0 + x] : c0 + x;
+      __syncthreads();  // the previous chunk's reads of Bs and sites (and at first the rows) are done
+      if (threadIdx.x < X) sites[x] = loc;
+      for (int col0 = cg; col0 < n; col0 += GM_CPT * CG) {
+        cplx<float> acc[GM_CPT][6];
+#pragma unroll
+        for (int cc = 0; cc < GM_CPT; cc++)
+#pragma unroll
+          for (int c = 0; c < 6; c++) acc[cc][c] = cplx<float>(0.f, 0.f);
+        if (in) {
+#pragma unroll 1
+          for (int k = d ? d - 1 : 0; k < (d ? d : 8); k++) {
+            const Nbr nb = neighbour(g, A, loc, k);
+            if (nb.cross != (d > 0)) continue;
+            const float sg = nb.flip ? 0.5f : -0.5f;
+#define GM_HOP(K)                                                                                                      \
+  case K: galerkin_hop<(K) / 2, ((K) & 1) == 0>(acc, P, U, sg, s, A, loc, nb.blk, nb.loc, nv, Vb, n, col0, CG); break;
+            switch (k) {
+              GM_HOP(0) GM_HOP(1) GM_HOP(2) GM_HOP(3) GM_HOP(4) GM_HOP(5) GM_HOP(6)
+              default: galerkin_hop<3, false>(acc, P, U, sg, s, A, loc, nb.blk, nb.loc, nv, Vb, n, col0, CG);
+            }
+#undef GM_HOP
+          }
+          if (d == 0) galerkin_site(acc, P, C.d + ((size_t)A * 36 + 18 * s) * Vb + loc, s, A, loc, nv, Vb, n, col0, CG);
+        }
+#pragma unroll
+        for (int cc = 0; cc < GM_CPT; cc++) {
+          const int col = col0 + cc * CG;
+          if (col < n)
+#pragma unroll
+            for (int c = 0; c < 6; c++) Bs[(size_t)col * BS + c * X + x] = make_float2(acc[cc][c].re, acc[cc][c].im);
+        }
+      }
+      __syncthreads();
+      // ---- projections: 4 sites of one component per instruction
+      if (warp < tiles) galerkin_tile<X>(cr0, ci0, Ps, Bs, sites, warp, ntile, nv, rs, Vb, lane);
+      if (warp + GM_THREADS / 32 < tiles)
+        galerkin_tile<X>(cr1, ci1, Ps, Bs, sites, warp + GM_THREADS / 32, ntile, nv, rs, Vb, lane);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+      const int tile = warp + q * (GM_THREADS / 32), mt = tile / ntile, nt = tile - mt * ntile;
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int row = mt * 16 + (lane >> 2) + (k >> 1) * 8, col = nt * 8 + 2 * (lane & 3) + (k & 1);
+        if (tile < tiles && row < nv && col < n)
+          Dc[(((size_t)A * 9 + d) * n + col) * n + s * nv + row] = q ? make_float2(cr1[k], ci1[k]) : make_float2(cr0[k], ci0[k]);
+      }
+    }
+  }
+}
+
+// words per row of P in shared memory: rows 4 banks apart
+static int galerkin_mma_rs(const FineGeom& g) { return (6 * g.Vb + 31) / 32 * 32 + 4; }
+static size_t galerkin_mma_smem(const FineGeom& g, int nv, int X) {
+  return (size_t)nv * galerkin_mma_rs(g) * 4 + (size_t)2 * nv * (6 * X + 4) * sizeof(float2);
+}
+template <int X>
+static bool try_galerkin_mma(const FineGeom& g, float2* Dc, const float2* P, Links<PREC_F32> U, Clover<PREC_F32> C, Geo q,
+                             FaceTables f, int nv, cudaStream_t st) {
+  const size_t smem = galerkin_mma_smem(g, nv, X);
+  if (smem > 226 * 1024 || (nv + 15) / 16 * ((2 * nv + 7) / 8) > 2 * (GM_THREADS / 32)) return false;
+  set_dynamic_smem((const void*)k_galerkin_mma<X>, smem);
+  k_galerkin_mma<X><<<g.Nb * 2, GM_THREADS, smem, st>>>(Dc, P, U, C, q, f, nv, galerkin_mma_rs(g));
+  return true;
+}
+
 static size_t galerkin_rows_smem(const FineGeom& g, const FaceDev& faces, int nv, int cc) {
   return (size_t)nv * 6 * g.Vb * sizeof(__half2) + (size_t)cc * 6 * (g.Vb + faces.off[8]) * sizeof(cplx<float>);
 }
@@ -287,7 +504,10 @@ void launch_galerkin(const FineGeom& g, const FaceDev& faces, int dprec, void* D
   Clover<PREC_F32> C{(const float2*)clover32, g.Vb};
   if (dprec != PREC_F32) throw Error(DDTM_ERR_ARG, "internal: Galerkin output is FP32");
   const size_t srows1 = galerkin_rows_smem(g, faces, nv, 1), srows2 = galerkin_rows_smem(g, faces, nv, 2);
-  if (rows_fp16 && srows2 <= 224 * 1024) {  // two columns per pass where the shared memory holds them
+  // matrix instructions with the widest chunk whose rows and columns fit in shared memory
+  if (rows_fp16 && (try_galerkin_mma<32>(g, (float2*)Dc, P, U, C, q, f, nv, st) || try_galerkin_mma<16>(g, (float2*)Dc, P, U, C, q, f, nv, st) ||
+                    try_galerkin_mma<8>(g, (float2*)Dc, P, U, C, q, f, nv, st))) {
+  } else if (rows_fp16 && srows2 <= 224 * 1024) {  // two columns per pass where the shared memory holds them
     set_dynamic_smem((const void*)k_galerkin_rows<2>, srows2);
     k_galerkin_rows<2><<<g.Nb * 2, threads, srows2, st>>>((float2*)Dc, P, U, C, q, f, nv);
   } else if (rows_fp16 && srows1 <= 220 * 1024) {
