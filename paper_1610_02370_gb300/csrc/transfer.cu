@@ -104,6 +104,139 @@ __global__ void k_build_P(float2* __restrict__ P, const float2* __restrict__ tv,
   }
 }
 
+// The same orthonormalisation, operation for operation, with the finished vectors kept on chip: the first ns of
+// them in shared memory, the rest (up to NR) in registers; each thread only ever reads its own site, so the
+// 4 i vector reads that orthogonalising vector i takes never leave the SM.  One CTA of 256 threads per SM.
+// 16^3 x 32, 24 vectors, 4^4 aggregates: 1.73 ms, k_build_P 2.34 ms, which is bound by 14 GB of L2 reads.  Bound by the
+// latency of the sequential Gram-Schmidt at 8 warps per SM (with a warp reduction per value and FP64 square roots in
+// every thread it took 2.00 ms).
+__device__ __forceinline__ void bp_dot(const float2 v[6], const float2 vi[6], float& pr, float& pi) {
+  pr = pi = 0.f;
+#pragma unroll
+  for (int comp = 0; comp < 6; comp++) {
+    pr += v[comp].x * vi[comp].x + v[comp].y * vi[comp].y;
+    pi += v[comp].x * vi[comp].y - v[comp].y * vi[comp].x;
+  }
+}
+__device__ __forceinline__ void bp_sub(float2 vi[6], float2 h, const float2 v[6]) {
+#pragma unroll
+  for (int comp = 0; comp < 6; comp++) {
+    vi[comp].x -= h.x * v[comp].x - h.y * v[comp].y;
+    vi[comp].y -= h.x * v[comp].y + h.y * v[comp].x;
+  }
+}
+// Warp sums of eight values at once: lanes with lane % 4 == 0 return the sum of value lane / 4's bits reversed,
+// idx = (lane & 16 ? 4 : 0) + (lane & 8 ? 2 : 0) + (lane & 4 ? 1 : 0); 9 shuffles instead of 40.
+__device__ __forceinline__ float warp_sum8(const float v[8], int lane) {
+  float a[4], b[2];
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const float send = lane & 16 ? v[k] : v[k + 4], keep = lane & 16 ? v[k + 4] : v[k];
+    a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; k++) {
+    const float send = lane & 8 ? a[k] : a[k + 2], keep = lane & 8 ? a[k + 2] : a[k];
+    b[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+  const float send = lane & 4 ? b[0] : b[1], keep = lane & 4 ? b[1] : b[0];
+  float c = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+template <int NR>
+__global__ void __launch_bounds__(256, 1) k_build_P_chip(float2* __restrict__ P, const float2* __restrict__ tv, int nv, int ns,
+                                                         int Vb, long V) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* vs = reinterpret_cast<float2*>(smem_raw);  // [ns][6][Vb]
+  __shared__ float red[8][2 * 72];                   // per warp, per vector; the norms in the last column
+  __shared__ float2 hco[72];
+  __shared__ float inv_sh;
+  const int blk = blockIdx.x >> 1, s = blockIdx.x & 1;
+  const int loc = threadIdx.x, lane = loc & 31, w = loc >> 5, nw = blockDim.x >> 5;
+  const int vidx = (lane & 16 ? 4 : 0) + (lane & 8 ? 2 : 0) + (lane & 4 ? 1 : 0);
+  const bool act = loc < Vb;
+  float2 vr[NR][6];
+#pragma unroll
+  for (int q = 0; q < NR; q++)
+#pragma unroll
+    for (int comp = 0; comp < 6; comp++) vr[q][comp] = make_float2(0.f, 0.f);
+  for (int i = 0; i < nv; i++) {
+    float2 vi[6];
+#pragma unroll
+    for (int comp = 0; comp < 6; comp++)
+      vi[comp] = act ? tv[(size_t)i * 12 * V + ((size_t)blk * 12 + 6 * s + comp) * Vb + loc] : make_float2(0.f, 0.f);
+    const int is = i < ns ? i : ns;  // finished vectors in shared memory
+    for (int pass = 0; pass < 2 && i > 0; pass++) {
+      // inner products, four vectors at a time
+      for (int j0 = 0; j0 < is; j0 += 4) {
+        float d[8];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          const int j = j0 + u < is ? j0 + u : is - 1;
+          float2 v[6];
+#pragma unroll
+          for (int comp = 0; comp < 6; comp++) v[comp] = act ? vs[(j * 6 + comp) * Vb + loc] : make_float2(0.f, 0.f);
+          bp_dot(v, vi, d[2 * u], d[2 * u + 1]);
+        }
+        const float t = warp_sum8(d, lane);
+        if ((lane & 3) == 0 && j0 + (vidx >> 1) < is) red[w][2 * j0 + vidx] = t;
+      }
+#pragma unroll
+      for (int q0 = 0; q0 < NR; q0 += 4)
+        if (ns + q0 < i) {
+          float d[8];
+#pragma unroll
+          for (int u = 0; u < 4; u++) bp_dot(vr[q0 + u], vi, d[2 * u], d[2 * u + 1]);
+          const float t = warp_sum8(d, lane);
+          if ((lane & 3) == 0) red[w][2 * (ns + q0) + vidx] = t;
+        }
+      __syncthreads();
+      for (int t = loc; t < 2 * i; t += blockDim.x) {  // t = 2 j: real part of <v_j, v_i>, 2 j + 1: imaginary part
+        double a = 0;
+        for (int k = 0; k < nw; k++) a += red[k][t];
+        reinterpret_cast<float*>(hco)[t] = (float)a;
+      }
+      __syncthreads();
+#pragma unroll 4
+      for (int j = 0; j < is; j++) {
+        float2 v[6];
+#pragma unroll
+        for (int comp = 0; comp < 6; comp++) v[comp] = act ? vs[(j * 6 + comp) * Vb + loc] : make_float2(0.f, 0.f);
+        bp_sub(vi, hco[j], v);
+      }
+#pragma unroll
+      for (int q = 0; q < NR; q++)
+        if (ns + q < i) bp_sub(vi, hco[ns + q], vr[q]);
+    }
+    float pn = 0;
+#pragma unroll
+    for (int comp = 0; comp < 6; comp++) pn += vi[comp].x * vi[comp].x + vi[comp].y * vi[comp].y;
+    pn = warp_sum(pn);
+    if (lane == 0) red[w][143] = pn;
+    __syncthreads();
+    if (loc == 0) {  // one thread: FP64 is slow here, and its pipe is shared by the whole SM
+      double nn = 0;
+      for (int k = 0; k < nw; k++) nn += red[k][143];
+      inv_sh = nn > 0 ? (float)(1.0 / sqrt(nn)) : 0.f;
+    }
+    __syncthreads();
+    const float inv = inv_sh;
+#pragma unroll
+    for (int comp = 0; comp < 6; comp++) {
+      vi[comp] = make_float2(vi[comp].x * inv, vi[comp].y * inv);
+      if (act) P[pidx(blk, s, i, comp, loc, nv, Vb)] = vi[comp];
+      if (act && i < ns) vs[(i * 6 + comp) * Vb + loc] = vi[comp];
+    }
+#pragma unroll
+    for (int q = 0; q < NR; q++)
+      if (ns + q == i) {
+#pragma unroll
+        for (int comp = 0; comp < 6; comp++) vr[q][comp] = vi[comp];
+      }
+  }
+}
+
 // Each CTA re-reads its aggregate half (nv x 6 x Vb complex FP32) from L2 in every Gram-Schmidt
 // step; when more CTAs run at once than L2 can hold the halves of, those re-reads go to HBM.  The
 // residency per SM is therefore capped (by reserving unused dynamic shared memory) so that the halves
@@ -118,6 +251,18 @@ static const size_t BP_L2_BYTES = (size_t)DDTM_BP_L2_MB << 20;
 void launch_build_P(const FineGeom& g, float2* P, const float2* tv, int nv, cudaStream_t st) {
   ScopedTimer timer_("build_P", st, nv);
   int threads = ((g.Vb + 31) / 32) * 32;
+  // on chip where the vectors fit: as many as shared memory holds, up to 16 more in registers (4^4 aggregates: up to 32
+  // vectors)
+  const size_t one = (size_t)6 * g.Vb * sizeof(float2);
+  const int ns = (int)(nv < (long)(216 * 1024 / one) ? nv : 216 * 1024 / one);
+  if (threads <= 256 && nv - ns <= 16) {
+    const void* k = nv - ns <= 8 ? (const void*)k_build_P_chip<8> : (const void*)k_build_P_chip<16>;
+    set_dynamic_smem(k, ns * one);
+    if (nv - ns <= 8) k_build_P_chip<8><<<g.Nb * 2, threads, ns * one, st>>>(P, tv, nv, ns, g.Vb, g.V);
+    else k_build_P_chip<16><<<g.Nb * 2, threads, ns * one, st>>>(P, tv, nv, ns, g.Vb, g.V);
+    CKL("build_P");
+    return;
+  }
   int dev = 0, sms = 0, smem_sm = 0, smem_blk = 0;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
