@@ -343,77 +343,86 @@ __global__ void k_restrict(cplx<float>* __restrict__ c, Spinor<PI> psi, size_t f
   }
 }
 
-// The same restriction with P read once per HC right-hand sides (the kernel
-// above reads it once per RC = 4): one CTA per block and chunk of HC
-// right-hand sides works through the
-// two chirality halves s in turn; for each it stages components 6s..6s+5 of the
-// chunk's block vectors in shared memory (FP32, [rc][6][Vb]: 72 KB for 6
-// right-hand sides at Vb = 256, so three CTAs share an SM), and warp w
-// computes OW outputs of half s at once (each staged entry read once serves OW outputs, each P entry HC
-// right-hand sides).  Every output is a sum over the block's 6 Vb entries in
-// the same order as k_restrict (lane partial sums over sites, then a warp sum).
-template <int PI, typename PS, int HC, int OW>
-__global__ void __launch_bounds__(256, 3) k_restrict_half(cplx<float>* __restrict__ c, Spinor<PI> psi, size_t fstride,
-                                                          long V, const PS* __restrict__ P, int nv, int R, int Rs) {
+// The same restriction for batches: one CTA per (block, chirality half s) and 2 NP right-hand sides, whose
+// block vectors it stages in shared memory as pairs ([pair][6][Vb], two right-hand sides per 16 bytes); warp w computes
+// OW outputs at once, both right-hand sides of a pair in packed f32x2 arithmetic.  Several sites' P entries are in
+// flight per lane: P comes from HBM once per 2 NP right-hand sides.  Every output is the same sum, in the same
+// order, as in k_restrict.
+template <int PI, typename PS, int NP, int OW, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_restrict_pair(cplx<float>* __restrict__ c, Spinor<PI> psi, size_t fstride, long V,
+                                                            const PS* __restrict__ P, int nv, int R, int Rs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* sp = reinterpret_cast<float2*>(smem_raw);  // [HC][6][Vb]
-  const int Vb = psi.Vb, blk = blockIdx.x, r0 = blockIdx.y * HC;
-  const int nr = R - r0 < HC ? R - r0 : HC;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int n = 2 * nv;
-  for (int s = 0; s < 2; s++) {
-    if (s) __syncthreads();  // the previous half's reads are done
-    for (int rc = 0; rc < HC; rc++) {
-      Spinor<PI> f = psi;
-      f.d += (size_t)(r0 + rc) * fstride;
-      if (f.nrm) f.nrm += (size_t)(r0 + rc) * V;
-      for (int loc = threadIdx.x; loc < Vb; loc += blockDim.x) {
-        if (rc < nr) {
-          cplx<typename Prec<PI>::real> v[12];
-          f.load(blk, loc, v);
+  float4* sp = reinterpret_cast<float4*>(smem_raw);
+  const int Vb = psi.Vb, nch = (R + 2 * NP - 1) / (2 * NP), bs = blockIdx.x / nch, r0 = (blockIdx.x - bs * nch) * 2 * NP;
+  const int blk = bs >> 1, s = bs & 1, lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = NT / 32, n = 2 * nv;
+  typedef typename Prec<PI>::store2 S;
+  for (int k = threadIdx.x; k < NP * Vb; k += NT) {
+    const int q = k / Vb, loc = k - q * Vb;
+    float4 v[6];
 #pragma unroll
-          for (int k = 0; k < 6; k++) {
-            const cplx<typename Prec<PI>::real> a = s ? v[6 + k] : v[k];  // constant register indices
-            sp[((size_t)rc * 6 + k) * Vb + loc] = make_float2((float)a.re, (float)a.im);
-          }
+    for (int l = 0; l < 2; l++) {
+      const int r = r0 + 2 * q + l < R ? r0 + 2 * q + l : R - 1;  // columns beyond R are not stored
+      const S* f = psi.d + (size_t)r * fstride + ((size_t)blk * 12 + 6 * s) * Vb + loc;
+      const typename Prec<PI>::real sc = Prec<PI>::scaled ? psi.nrm[(size_t)r * V + (size_t)blk * Vb + loc] : 1;
+#pragma unroll
+      for (int e = 0; e < 6; e++) {
+        auto z = ld(f + (size_t)e * Vb);
+        if (Prec<PI>::scaled) z = sc * z;
+        if (l) {
+          v[e].y = (float)z.re;
+          v[e].w = (float)z.im;
         } else {
-#pragma unroll
-          for (int k = 0; k < 6; k++) sp[((size_t)rc * 6 + k) * Vb + loc] = make_float2(0.f, 0.f);
+          v[e].x = (float)z.re;
+          v[e].z = (float)z.im;
         }
       }
     }
-    __syncthreads();
-    for (int i0 = w * OW; i0 < nv; i0 += nw * OW) {
-      cplx<float> acc[OW][HC];
 #pragma unroll
-      for (int u = 0; u < OW; u++)
+    for (int e = 0; e < 6; e++) sp[(q * 6 + e) * Vb + loc] = v[e];
+  }
+  __syncthreads();
+  for (int i0 = w * OW; i0 < nv; i0 += nw * OW) {
+    float2 re[OW][NP], im[OW][NP];
 #pragma unroll
-        for (int rc = 0; rc < HC; rc++) acc[u][rc] = cplx<float>(0, 0);
-      for (int comp = 0; comp < 6; comp++)
-        for (int loc = lane; loc < Vb; loc += 32) {
-          cplx<float> pv[OW];
+    for (int u = 0; u < OW; u++)
+#pragma unroll
+      for (int q = 0; q < NP; q++) re[u][q] = im[u][q] = make_float2(0.f, 0.f);
+    const PS* row[OW];
+#pragma unroll
+    for (int u = 0; u < OW; u++) row[u] = P + ((size_t)(blk * 2 + s) * nv + (i0 + u < nv ? i0 + u : nv - 1)) * 6 * Vb;
+    for (int comp = 0; comp < 6; comp++)
+#pragma unroll 8
+      for (int loc = lane; loc < Vb; loc += 32) {
+        float2 pr[OW], pi[OW], pn[OW];
+#pragma unroll
+        for (int u = 0; u < OW; u++) {
+          const cplx<float> pv = ldp<PS>(row[u] + comp * Vb + loc);
+          pr[u] = make_float2(pv.re, pv.re);
+          pi[u] = make_float2(pv.im, pv.im);
+          pn[u] = make_float2(-pv.im, -pv.im);
+        }
+#pragma unroll
+        for (int q = 0; q < NP; q++) {
+          const float4 y = sp[(q * 6 + comp) * Vb + loc];
+          const float2 yr = make_float2(y.x, y.y), yi = make_float2(y.z, y.w);
 #pragma unroll
           for (int u = 0; u < OW; u++) {
-            const int i = i0 + u < nv ? i0 + u : nv - 1;
-            pv[u] = ldp<PS>(P + (((size_t)(blk * 2 + s) * nv + i) * 6 + comp) * Vb + loc);
-          }
-#pragma unroll
-          for (int rc = 0; rc < HC; rc++) {
-            const float2 f2 = sp[((size_t)rc * 6 + comp) * Vb + loc];
-            const cplx<float> fv(f2.x, f2.y);
-#pragma unroll
-            for (int u = 0; u < OW; u++) cmac_conj(acc[u][rc], pv[u], fv);
+            re[u][q] = __ffma2_rn(pr[u], yr, __ffma2_rn(pi[u], yi, re[u][q]));
+            im[u][q] = __ffma2_rn(pr[u], yi, __ffma2_rn(pn[u], yr, im[u][q]));
           }
         }
+      }
 #pragma unroll
-      for (int u = 0; u < OW; u++)
+    for (int u = 0; u < OW; u++)
 #pragma unroll
-        for (int rc = 0; rc < HC; rc++) {
-          acc[u][rc].re = warp_sum(acc[u][rc].re);
-          acc[u][rc].im = warp_sum(acc[u][rc].im);
-          if (lane == 0 && rc < nr && i0 + u < nv) c[((size_t)blk * n + s * nv + i0 + u) * Rs + r0 + rc] = acc[u][rc];
+      for (int q = 0; q < NP; q++) {
+        const float a = warp_sum(re[u][q].x), b = warp_sum(im[u][q].x), d = warp_sum(re[u][q].y), e = warp_sum(im[u][q].y);
+        if (lane == 0 && i0 + u < nv) {
+          cplx<float>* o = c + ((size_t)blk * n + s * nv + i0 + u) * Rs + r0 + 2 * q;
+          if (r0 + 2 * q < R) o[0] = cplx<float>(a, b);
+          if (r0 + 2 * q + 1 < R) o[1] = cplx<float>(d, e);
         }
-    }
+      }
   }
 }
 
@@ -471,94 +480,112 @@ __global__ void k_prolong(Spinor<PO> x, size_t fstride, long V, const cplx<float
   }
 }
 
-// The same prolongation with P read once per HC right-hand sides (the kernel
-// above reads it once per PRO_RC = 2): one CTA per block and chunk of HC
-// right-hand sides, thread = site.  The 6 x HC components of chirality half
-// s = 0 are formed in registers and parked in shared memory ([HC][6][Vb],
-// each thread its own site), those of s = 1 are formed next, and the site's 12
-// components of each right-hand side are stored together (FP16 storage keeps
-// one scale per site).  Every component is the same sum, in the same order,
-// as in k_prolong, so the results are identical.
-template <int PO, typename PS, int HC>
-__global__ void __launch_bounds__(256, 2) k_prolong_half(Spinor<PO> x, size_t fstride, long V, const cplx<float>* __restrict__ e,
+// The same prolongation for batches: one CTA per block and 2 NP right-hand sides (neighbouring CTAs share the block's P
+// through L2), thread = site, right-hand sides in pairs of packed f32x2 arithmetic.  The components of chirality half
+// s = 0 are formed in registers and parked in shared memory ([NP][6][Vb] pairs, each thread its own site), those of s =
+// 1 are formed next, and the site's 12 components of each right-hand side are stored together (FP16 storage keeps one
+// scale per site).  The next vector's P entries are loaded while one is used.  Every component is the same sum, in
+// the same order, as in k_prolong.
+template <int PO, typename PS, int NP>
+__global__ void __launch_bounds__(256, 2) k_prolong_pair(Spinor<PO> x, size_t fstride, long V, const cplx<float>* __restrict__ e,
                                                          const PS* __restrict__ P, int nv, int R, int Rs, int add) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   typedef typename Prec<PO>::real Rl;
-  const int Vb = x.Vb, blk = blockIdx.x, n = 2 * nv, r0 = blockIdx.y * HC;
-  const int nr = R - r0 < HC ? R - r0 : HC;
-  float2* park = reinterpret_cast<float2*>(smem_raw);                       // [HC][6][Vb]
-  cplx<float>* se = reinterpret_cast<cplx<float>*>(park + (size_t)HC * 6 * Vb);  // [n][HC]
-  for (int k = threadIdx.x; k < n * HC; k += blockDim.x) {
-    const int o = k / HC, rc = k - o * HC;
-    se[k] = rc < nr ? e[((size_t)blk * n + o) * Rs + r0 + rc] : cplx<float>(0, 0);
+  const int Vb = x.Vb, n = 2 * nv, nch = (R + 2 * NP - 1) / (2 * NP), blk = blockIdx.x / nch, r0 = (blockIdx.x - blk * nch) * 2 * NP;
+  float4* park = reinterpret_cast<float4*>(smem_raw);   // [NP][6][Vb]
+  float4* se = park + (size_t)NP * 6 * Vb;               // [n][NP]
+  for (int k = threadIdx.x; k < n * NP; k += blockDim.x) {
+    const int o = k / NP, q = k - o * NP, r = r0 + 2 * q;
+    const cplx<float> a = r < R ? e[((size_t)blk * n + o) * Rs + r] : cplx<float>(0, 0);
+    const cplx<float> b = r + 1 < R ? e[((size_t)blk * n + o) * Rs + r + 1] : cplx<float>(0, 0);
+    se[k] = make_float4(a.re, b.re, a.im, b.im);
   }
   __syncthreads();
   for (int loc = threadIdx.x; loc < Vb; loc += blockDim.x) {
 #pragma unroll 1
     for (int s = 0; s < 2; s++) {
-      cplx<float> acc[HC][6];
+      float2 re[NP][6], im[NP][6];
 #pragma unroll
-      for (int rc = 0; rc < HC; rc++)
+      for (int q = 0; q < NP; q++)
 #pragma unroll
-        for (int c = 0; c < 6; c++) acc[rc][c] = cplx<float>(0, 0);
+        for (int c = 0; c < 6; c++) re[q][c] = im[q][c] = make_float2(0.f, 0.f);
+      const PS* col = P + (size_t)(blk * 2 + s) * nv * 6 * Vb + loc;
+      cplx<float> pv[6], nx[6];
+#pragma unroll
+      for (int c = 0; c < 6; c++) nx[c] = ldp<PS>(col + (size_t)c * Vb);
+#pragma unroll 2
       for (int i = 0; i < nv; i++) {
-        const PS* col = P + ((size_t)(blk * 2 + s) * nv + i) * 6 * Vb + loc;
-        cplx<float> pv[6];
 #pragma unroll
-        for (int c = 0; c < 6; c++) pv[c] = ldp<PS>(col + (size_t)c * Vb);
+        for (int c = 0; c < 6; c++) pv[c] = nx[c];
+        const PS* nc = col + (size_t)(i + 1 < nv ? i + 1 : i) * 6 * Vb;
 #pragma unroll
-        for (int rc = 0; rc < HC; rc++) {
-          const cplx<float> ev = se[(s * nv + i) * HC + rc];
+        for (int c = 0; c < 6; c++) nx[c] = ldp<PS>(nc + (size_t)c * Vb);
 #pragma unroll
-          for (int c = 0; c < 6; c++) cmac(acc[rc][c], pv[c], ev);
+        for (int q = 0; q < NP; q++) {
+          const float4 ev = se[(s * nv + i) * NP + q];
+          const float2 er = make_float2(ev.x, ev.y), ei = make_float2(ev.z, ev.w);
+#pragma unroll
+          for (int c = 0; c < 6; c++) {
+            const float2 pr = make_float2(pv[c].re, pv[c].re), pi = make_float2(pv[c].im, pv[c].im),
+                         pn = make_float2(-pv[c].im, -pv[c].im);
+            re[q][c] = __ffma2_rn(pr, er, __ffma2_rn(pn, ei, re[q][c]));
+            im[q][c] = __ffma2_rn(pr, ei, __ffma2_rn(pi, er, im[q][c]));
+          }
         }
       }
       if (s == 0) {
 #pragma unroll
-        for (int rc = 0; rc < HC; rc++)
+        for (int q = 0; q < NP; q++)
 #pragma unroll
-          for (int c = 0; c < 6; c++) park[((size_t)rc * 6 + c) * Vb + loc] = make_float2(acc[rc][c].re, acc[rc][c].im);
+          for (int c = 0; c < 6; c++) park[((size_t)q * 6 + c) * Vb + loc] = make_float4(re[q][c].x, re[q][c].y, im[q][c].x, im[q][c].y);
       } else {
 #pragma unroll
-        for (int rc = 0; rc < HC; rc++) {
-          if (rc >= nr) break;
-          Spinor<PO> f = x;
-          f.d += (size_t)(r0 + rc) * fstride;
-          if (f.nrm) f.nrm += (size_t)(r0 + rc) * V;
-          cplx<Rl> out[12];
-          if (add) f.loadw(blk, loc, out);
+        for (int q = 0; q < NP; q++)
 #pragma unroll
-          for (int k = 0; k < 12; k++) {
-            cplx<float> a;
-            if (k < 6) {
-              const float2 v = park[((size_t)rc * 6 + k) * Vb + loc];
-              a = cplx<float>(v.x, v.y);
-            } else {
-              a = acc[rc][k - 6];
+          for (int l = 0; l < 2; l++) {
+            const int r = r0 + 2 * q + l;
+            if (r >= R) break;
+            Spinor<PO> f = x;
+            f.d += (size_t)r * fstride;
+            if (f.nrm) f.nrm += (size_t)r * V;
+            cplx<Rl> out[12];
+            if (add) f.loadw(blk, loc, out);
+#pragma unroll
+            for (int k = 0; k < 12; k++) {
+              cplx<float> a;
+              if (k < 6) {
+                const float4 v = park[((size_t)q * 6 + k) * Vb + loc];
+                a = l ? cplx<float>(v.y, v.w) : cplx<float>(v.x, v.z);
+              } else {
+                a = l ? cplx<float>(re[q][k - 6].y, im[q][k - 6].y) : cplx<float>(re[q][k - 6].x, im[q][k - 6].x);
+              }
+              const cplx<Rl> ar((Rl)a.re, (Rl)a.im);
+              out[k] = add ? out[k] + ar : ar;
             }
-            const cplx<Rl> ar((Rl)a.re, (Rl)a.im);
-            out[k] = add ? out[k] + ar : ar;
+            f.store(blk, loc, out);
           }
-          f.store(blk, loc, out);
-        }
       }
     }
   }
 }
 
 static const int RST_RC = 4, PRO_RC = 2;
-static const int PH_C = 6;  // right-hand sides per CTA of k_prolong_half
+static const int PP_NP = 3;  // pairs per CTA of k_prolong_pair
 
-static const int RH_C = 6, RH_OW = 3;  // right-hand sides per CTA, outputs per warp pass
+// k_restrict_pair: pairs per CTA, outputs per warp pass, threads, CTAs per SM.  24^3 x 48, 12 right-hand sides, 24
+// vectors, FP32: 3, 3, 256, 2: 532 us; 3, 3, 256, 3: 667; 3, 2, 384, 2: 550; 6, 2, 384, 1: 616; 6, 1, 768, 1: 718
+// (scalar arithmetic, two P entries in flight and the chunks of a block far apart: 1025).  The prolongation, 3 pairs:
+// 561 us (815).  Both are bound by the latency of the P loads and shared memory; P and the fields alone take 340 us.
+static const int RP_NP = 3, RP_OW = 3, RP_NT = 256, RP_MINB = 2;
 template <int PI, typename PS>
 static void restrict_p(const FineGeom& g, cplx<float>* c, Spinor<PI> f, size_t fstride, const PS* P, int nv, int R,
                        int Rs, cudaStream_t st) {
-  if (R > RST_RC && (size_t)RH_C * 6 * g.Vb * sizeof(float2) <= 200 * 1024) {
-    // several chunks of RST_RC would read P once per chunk: read it once per RH_C right-hand sides
-    const size_t smem = (size_t)RH_C * 6 * g.Vb * sizeof(float2);
-    set_dynamic_smem((const void*)k_restrict_half<PI, PS, RH_C, RH_OW>, smem);
-    dim3 grid(g.Nb, (R + RH_C - 1) / RH_C);
-    k_restrict_half<PI, PS, RH_C, RH_OW><<<grid, 256, smem, st>>>(c, f, fstride, g.V, P, nv, R, Rs);
+  const size_t psmem = (size_t)RP_NP * 6 * g.Vb * sizeof(float4);
+  if (R > RST_RC && psmem <= 200 * 1024) {
+    // several chunks of RST_RC would read P once per chunk: read it once per 2 RP_NP right-hand sides
+    set_dynamic_smem((const void*)k_restrict_pair<PI, PS, RP_NP, RP_OW, RP_NT, RP_MINB>, psmem);
+    const unsigned grid = (unsigned)g.Nb * 2 * ((R + 2 * RP_NP - 1) / (2 * RP_NP));
+    k_restrict_pair<PI, PS, RP_NP, RP_OW, RP_NT, RP_MINB><<<grid, RP_NT, psmem, st>>>(c, f, fstride, g.V, P, nv, R, Rs);
     return;
   }
   size_t smem = (size_t)RST_RC * 12 * g.Vb * sizeof(cplx<float>);
@@ -578,12 +605,12 @@ static void restrict_t(const FineGeom& g, int pin, cplx<float>* c, const void* p
 }
 
 template <int PO, typename PS>
-static void prolong_half_p(const FineGeom& g, Spinor<PO> x, size_t fs, const cplx<float>* e, const PS* P, int nv, int R,
+static void prolong_pair_p(const FineGeom& g, Spinor<PO> x, size_t fs, const cplx<float>* e, const PS* P, int nv, int R,
                            int Rs, int add, size_t smem, cudaStream_t st) {
-  set_dynamic_smem((const void*)k_prolong_half<PO, PS, PH_C>, smem);
-  dim3 grid(g.Nb, (R + PH_C - 1) / PH_C);
+  set_dynamic_smem((const void*)k_prolong_pair<PO, PS, PP_NP>, smem);
+  const unsigned grid = (unsigned)g.Nb * ((R + 2 * PP_NP - 1) / (2 * PP_NP));
   const int threads = g.Vb < 256 ? ((g.Vb + 31) / 32) * 32 : 256;
-  k_prolong_half<PO, PS, PH_C><<<grid, threads, smem, st>>>(x, fs, g.V, e, P, nv, R, Rs, add);
+  k_prolong_pair<PO, PS, PP_NP><<<grid, threads, smem, st>>>(x, fs, g.V, e, P, nv, R, Rs, add);
 }
 
 template <typename PS>
@@ -592,13 +619,13 @@ static void prolong_t(const FineGeom& g, int pout, void* x, float* xn, const cpl
   size_t smem = (size_t)2 * nv * Rs * sizeof(cplx<float>);
   int threads = g.Vb < 128 ? ((g.Vb + 31) / 32) * 32 : 128;
   size_t fs = (size_t)g.V * 12;
-  const size_t hsmem = (size_t)PH_C * 6 * g.Vb * sizeof(float2) + (size_t)2 * nv * PH_C * sizeof(cplx<float>);
+  const size_t hsmem = (size_t)PP_NP * 6 * g.Vb * sizeof(float4) + (size_t)2 * nv * PP_NP * sizeof(float4);
   if (R > PRO_RC && pout != PREC_F64 && hsmem <= 100 * 1024) {
-    // several chunks of PRO_RC would read P once per chunk: read it once per PH_C right-hand sides
+    // several chunks of PRO_RC would read P once per chunk: read it once per 2 PP_NP right-hand sides
     if (pout == PREC_F32)
-      prolong_half_p<PREC_F32, PS>(g, Spinor<PREC_F32>{(float2*)x, nullptr, g.Vb}, fs, e, P, nv, R, Rs, add, hsmem, st);
+      prolong_pair_p<PREC_F32, PS>(g, Spinor<PREC_F32>{(float2*)x, nullptr, g.Vb}, fs, e, P, nv, R, Rs, add, hsmem, st);
     else
-      prolong_half_p<PREC_F16, PS>(g, Spinor<PREC_F16>{(__half2*)x, xn, g.Vb}, fs, e, P, nv, R, Rs, add, hsmem, st);
+      prolong_pair_p<PREC_F16, PS>(g, Spinor<PREC_F16>{(__half2*)x, xn, g.Vb}, fs, e, P, nv, R, Rs, add, hsmem, st);
     CKL("prolong");
     return;
   }
@@ -614,17 +641,238 @@ static void prolong_t(const FineGeom& g, int pout, void* x, float* xn, const cpl
   CKL("prolong");
 }
 
+// ---- restriction and prolongation of FP16 fields with the FP16 copy of P (the smoother's precision) -----------
+// Both are dense contractions per aggregate and chirality half s, with R right-hand sides as columns:
+//   c[i][r] = sum over (component, site) conj(P_i) psi_r        (nv x R, depth 6 Vb)
+//   x_r(component, site) = sum_i P_i e[i][r]                    (6 Vb x R, depth nv)
+// done by mma.sync m16n8k8 in TF32: P's FP16 entries are exact in TF32, the other operand goes in as hi + lo (21 bits),
+// sums are FP32.  The unit's sums carry about 2e-6 (measured with FP32 operands in three products, against 3e-7 of
+// the FP32 kernels above, which therefore keep FP32 fields); beside the 5e-4 of the FP16 operands that is nothing.
+// Fragments are loaded straight from memory: P once per 16 right-hand sides, psi once.  A complex product takes 4 of
+// the 8 depths for the real and 4 for the imaginary parts.  Every right-hand side is a column of its own, so a batch
+// gives the same bits as its right-hand sides one by one.
+// 16^3 x 32, 12 right-hand sides, 24 vectors: restriction 135 us, prolongation 161 us (SIMT kernels above 292, 202).
+__device__ __forceinline__ uint32_t tf32_of(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ uint32_t neg_u(uint32_t x) { return x ^ 0x80000000u; }
+__device__ __forceinline__ void mma_t(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// a fragment of A: FP16 complex entries of rows g and g + 8, one k each
+struct AFrag {
+  uint32_t gr, gi, hr, hi;
+};
+__device__ __forceinline__ AFrag a_frag(cplx<float> g, cplx<float> h) {
+  return AFrag{__float_as_uint(g.re), __float_as_uint(g.im), __float_as_uint(h.re), __float_as_uint(h.im)};
+}
+// a fragment of B: one complex entry as hi + lo
+struct BFrag {
+  uint32_t re, im, rel, iml;
+};
+__device__ __forceinline__ BFrag b_frag(cplx<float> z) {
+  BFrag f;
+  f.re = tf32_of(z.re);
+  f.im = tf32_of(z.im);
+  f.rel = tf32_of(z.re - __uint_as_float(f.re));
+  f.iml = tf32_of(z.im - __uint_as_float(f.im));
+  return f;
+}
+// (cr, ci) += conj(A) B (CONJ) or A B
+template <bool CONJ>
+__device__ __forceinline__ void cmma(float (&cr)[4], float (&ci)[4], const AFrag& a, const BFrag& b) {
+  const uint32_t ngi = neg_u(a.gi), nhi = neg_u(a.hi);
+  if (CONJ) {  // re: ar br + ai bi; im: -ai br + ar bi
+    mma_t(cr, a.gr, a.hr, a.gi, a.hi, b.re, b.im);
+    mma_t(ci, ngi, nhi, a.gr, a.hr, b.re, b.im);
+    mma_t(cr, a.gr, a.hr, a.gi, a.hi, b.rel, b.iml);
+    mma_t(ci, ngi, nhi, a.gr, a.hr, b.rel, b.iml);
+  } else {  // re: ar br - ai bi; im: ai br + ar bi
+    mma_t(cr, a.gr, a.hr, ngi, nhi, b.re, b.im);
+    mma_t(ci, a.gi, a.hi, a.gr, a.hr, b.re, b.im);
+    mma_t(cr, a.gr, a.hr, ngi, nhi, b.rel, b.iml);
+    mma_t(ci, a.gi, a.hi, a.gr, a.hr, b.rel, b.iml);
+  }
+}
+
+// c = P^dagger psi.  One CTA per (aggregate, s) and 8 NT right-hand sides; its warps share the depth (runs of 4 sites
+// of a component), every warp forms all rows, and the partial sums meet in shared memory.
+static const int RM_WARPS = 12;
+template <int MT, int NT>
+__global__ void __launch_bounds__(32 * RM_WARPS) k_restrict_mma(cplx<float>* __restrict__ c, Spinor<PREC_F16> psi, size_t fstride, long V,
+                                                               const __half2* __restrict__ P, int nv, int R, int Rs) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* part = reinterpret_cast<float2*>(smem_raw);  // [warp][16 MT][8 NT + 1]
+  const int Vb = psi.Vb, blk = blockIdx.x >> 1, s = blockIdx.x & 1, r0 = blockIdx.y * 8 * NT;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  float cr[MT][NT][4], ci[MT][NT][4];
+#pragma unroll
+  for (int m = 0; m < MT; m++)
+#pragma unroll
+    for (int q = 0; q < NT; q++)
+#pragma unroll
+      for (int k = 0; k < 4; k++) cr[m][q][k] = ci[m][q][k] = 0.f;
+  const __half2* pg[MT];
+  const __half2* ph[MT];
+#pragma unroll
+  for (int m = 0; m < MT; m++) {  // rows beyond nv repeat the last one and are not stored
+    const int i0 = 16 * m + g < nv ? 16 * m + g : nv - 1, i1 = 16 * m + g + 8 < nv ? 16 * m + g + 8 : nv - 1;
+    pg[m] = P + ((size_t)(blk * 2 + s) * nv + i0) * 6 * Vb + t;
+    ph[m] = P + ((size_t)(blk * 2 + s) * nv + i1) * 6 * Vb + t;
+  }
+  const __half2* f[NT];
+  const float* fn[NT];
+#pragma unroll
+  for (int q = 0; q < NT; q++) {  // columns beyond R repeat the last one
+    const int r = r0 + 8 * q + g < R ? r0 + 8 * q + g : R - 1;
+    f[q] = psi.d + (size_t)r * fstride + ((size_t)blk * 12 + 6 * s) * Vb + t;
+    fn[q] = psi.nrm + (size_t)r * V + (size_t)blk * Vb + t;
+  }
+  const int ks = 6 * Vb / 4, kb = warp * ks / RM_WARPS, ke = (warp + 1) * ks / RM_WARPS;
+  int site = 4 * kb % Vb;
+#pragma unroll 4
+  for (int k = kb; k < ke; k++) {
+    const int e = 4 * k;  // component * Vb + site of the run
+    BFrag b[NT];
+#pragma unroll
+    for (int q = 0; q < NT; q++) {
+      b[q] = b_frag(__ldg(fn[q] + site) * ld(f[q] + e));
+    }
+#pragma unroll
+    for (int m = 0; m < MT; m++) {
+      const AFrag a = a_frag(ld(pg[m] + e), ld(ph[m] + e));
+#pragma unroll
+      for (int q = 0; q < NT; q++) cmma<true>(cr[m][q], ci[m][q], a, b[q]);
+    }
+    site = site + 4 < Vb ? site + 4 : 0;
+  }
+  constexpr int LD = 8 * NT + 1;
+#pragma unroll
+  for (int m = 0; m < MT; m++)
+#pragma unroll
+    for (int q = 0; q < NT; q++)
+#pragma unroll
+      for (int k = 0; k < 4; k++)
+        part[((size_t)warp * 16 * MT + 16 * m + g + 8 * (k >> 1)) * LD + 8 * q + 2 * t + (k & 1)] = make_float2(cr[m][q][k], ci[m][q][k]);
+  __syncthreads();
+  for (int o = threadIdx.x; o < 16 * MT * 8 * NT; o += blockDim.x) {
+    const int i = o / (8 * NT), r = o - i * 8 * NT;
+    if (i >= nv || r0 + r >= R) continue;
+    float re = 0.f, im = 0.f;
+#pragma unroll
+    for (int w = 0; w < RM_WARPS; w++) {
+      const float2 p = part[((size_t)w * 16 * MT + i) * LD + r];
+      re += p.x;
+      im += p.y;
+    }
+    c[((size_t)blk * 2 * nv + s * nv + i) * Rs + r0 + r] = cplx<float>(re, im);
+  }
+}
+
+// x_r = P e_r (add = 0) or x_r += P e_r.  One CTA per aggregate and 8 right-hand sides (neighbouring CTAs share the
+// aggregate's P through L2); a warp takes 16 sites at a time and all 12 components of them (FP16 storage keeps
+// one scale per site), e_B comes from shared memory.
+__global__ void __launch_bounds__(128, 3) k_prolong_mma(Spinor<PREC_F16> x, size_t fstride, long V, const cplx<float>* __restrict__ e,
+                                                        const __half2* __restrict__ P, int nv, int R, int Rs, int add) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* se = reinterpret_cast<float2*>(smem_raw);  // [2][nv4][9], rows beyond nv are zero
+  const int Vb = x.Vb, nchunk = (R + 7) / 8, blk = blockIdx.x / nchunk, r0 = (blockIdx.x - blk * nchunk) * 8;
+  const int nv4 = (nv + 3) / 4 * 4, n = 2 * nv;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, nw = blockDim.x >> 5;
+  for (int k = threadIdx.x; k < 2 * nv4 * 8; k += blockDim.x) {
+    const int r = k & 7, o = k >> 3, s = o / nv4, i = o - s * nv4;
+    const cplx<float> z = i < nv && r0 + r < R ? e[((size_t)blk * n + s * nv + i) * Rs + r0 + r] : cplx<float>(0, 0);
+    se[o * 9 + r] = make_float2(z.re, z.im);
+  }
+  __syncthreads();
+  for (int x0 = 16 * warp; x0 < Vb; x0 += 16 * nw) {
+    float cr[12][4], ci[12][4];
+#pragma unroll
+    for (int c = 0; c < 12; c++)
+#pragma unroll
+      for (int k = 0; k < 4; k++) cr[c][k] = ci[c][k] = 0.f;
+#pragma unroll
+    for (int s = 0; s < 2; s++)
+#pragma unroll 1
+      for (int i0 = 0; i0 < nv; i0 += 4) {
+        const float2 ev = se[(s * nv4 + i0 + t) * 9 + g];
+        const BFrag b = b_frag(cplx<float>(ev.x, ev.y));
+        const int i = i0 + t < nv ? i0 + t : nv - 1;  // beyond nv e is zero
+        const __half2* p = P + ((size_t)(blk * 2 + s) * nv + i) * 6 * Vb + x0 + g;
+        cplx<float> pa[6], pb[6];
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+          pa[c] = ld(p + (size_t)c * Vb);
+          pb[c] = ld(p + (size_t)c * Vb + 8);
+        }
+#pragma unroll
+        for (int c = 0; c < 6; c++) cmma<false>(cr[6 * s + c], ci[6 * s + c], a_frag(pa[c], pb[c]), b);
+      }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      const int r = r0 + 2 * t + (k & 1), loc = x0 + g + 8 * (k >> 1);
+      if (r >= R) continue;
+      Spinor<PREC_F16> f = x;
+      f.d += (size_t)r * fstride;
+      f.nrm += (size_t)r * V;
+      cplx<float> out[12];
+      if (add) f.loadw(blk, loc, out);
+#pragma unroll
+      for (int c = 0; c < 12; c++) {
+        const cplx<float> a(cr[c][k], ci[c][k]);
+        out[c] = add ? out[c] + a : a;
+      }
+      f.store(blk, loc, out);
+    }
+  }
+}
+
+template <int MT>
+static void restrict_mma_m(const FineGeom& g, cplx<float>* c, Spinor<PREC_F16> f, const __half2* P, int nv, int R, int Rs, cudaStream_t st) {
+  const int NT = R <= 8 ? 1 : 2;
+  const size_t smem = (size_t)RM_WARPS * 16 * MT * (8 * NT + 1) * sizeof(float2);
+  const void* k = NT == 1 ? (const void*)k_restrict_mma<MT, 1> : (const void*)k_restrict_mma<MT, 2>;
+  set_dynamic_smem(k, smem);
+  const dim3 grid(g.Nb * 2, (R + 8 * NT - 1) / (8 * NT));
+  if (NT == 1) k_restrict_mma<MT, 1><<<grid, 32 * RM_WARPS, smem, st>>>(c, f, (size_t)g.V * 12, g.V, P, nv, R, Rs);
+  else k_restrict_mma<MT, 2><<<grid, 32 * RM_WARPS, smem, st>>>(c, f, (size_t)g.V * 12, g.V, P, nv, R, Rs);
+  CKL("restrict");
+}
+static void restrict_mma(const FineGeom& g, cplx<float>* c, const void* psi, const float* pn, const __half2* P, int nv, int R, int Rs,
+                         cudaStream_t st) {
+  const Spinor<PREC_F16> f{(__half2*)psi, (float*)pn, g.Vb};
+  if (nv <= 16) restrict_mma_m<1>(g, c, f, P, nv, R, Rs, st);
+  else if (nv <= 32) restrict_mma_m<2>(g, c, f, P, nv, R, Rs, st);
+  else restrict_mma_m<4>(g, c, f, P, nv, R, Rs, st);
+}
+static void prolong_mma(const FineGeom& g, void* x, float* xn, const cplx<float>* e, const __half2* P, int nv, int R, int Rs, int add,
+                        cudaStream_t st) {
+  const size_t smem = (size_t)2 * ((nv + 3) / 4 * 4) * 9 * sizeof(float2);
+  const int threads = g.Vb < 64 ? 2 * g.Vb : 128;  // a warp per 16 sites, four at most
+  k_prolong_mma<<<(unsigned)g.Nb * ((R + 7) / 8), threads, smem, st>>>(Spinor<PREC_F16>{(__half2*)x, xn, g.Vb}, (size_t)g.V * 12,
+                                                                      g.V, e, P, nv, R, Rs, add);
+  CKL("prolong");
+}
+
 void launch_restrict(const FineGeom& g, int pin, cplx<float>* c, const void* psi, const float* pn, const void* P,
                      int pprec, int nv, int R, int Rs, cudaStream_t st) {
   ScopedTimer timer_(pin == PREC_F16 ? "restrict_f16" : pin == PREC_F32 ? "restrict_f32" : "restrict_f64", st, R);
-  if (pprec == PREC_F16) restrict_t<__half2>(g, pin, c, psi, pn, (const __half2*)P, nv, R, Rs, st);
+  if (R <= 0) return;
+  if (pprec == PREC_F16 && pin == PREC_F16) restrict_mma(g, c, psi, pn, (const __half2*)P, nv, R, Rs, st);
+  else if (pprec == PREC_F16) restrict_t<__half2>(g, pin, c, psi, pn, (const __half2*)P, nv, R, Rs, st);
   else restrict_t<float2>(g, pin, c, psi, pn, (const float2*)P, nv, R, Rs, st);
 }
 
 void launch_prolong(const FineGeom& g, int pout, void* x, float* xn, const cplx<float>* e, const void* P, int pprec,
                     int nv, int R, int Rs, int add, cudaStream_t st) {
   ScopedTimer timer_(pout == PREC_F16 ? "prolong_f16" : pout == PREC_F32 ? "prolong_f32" : "prolong_f64", st, R);
-  if (pprec == PREC_F16) prolong_t<__half2>(g, pout, x, xn, e, (const __half2*)P, nv, R, Rs, add, st);
+  if (R <= 0) return;
+  if (pprec == PREC_F16 && pout == PREC_F16) prolong_mma(g, x, xn, e, (const __half2*)P, nv, R, Rs, add, st);
+  else if (pprec == PREC_F16) prolong_t<__half2>(g, pout, x, xn, e, (const __half2*)P, nv, R, Rs, add, st);
   else prolong_t<float2>(g, pout, x, xn, e, (const float2*)P, nv, R, Rs, add, st);
 }
 
