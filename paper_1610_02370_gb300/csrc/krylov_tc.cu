@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(NT, 1) k_gs_step(const GsArgs a) {
   const bool single = ntiles <= W / a.ngj;  // at most one tile per slot: w stays in registers
   // right-hand side whose Givens update this warp does (-1: none): warps from the last one down
   const int my_r = blockIdx.x + G * (NW - 1 - warp) < R ? (int)blockIdx.x + G * (NW - 1 - warp) : -1;
+  const bool idle = t0 >= ntiles;  // no tile: the Givens column can be turned while the other warps update theirs
   float2* hs = reinterpret_cast<float2*>(smem_raw);  // [slot][GS_CHUNK][4], later [GS_CHUNK][4 ngj]
   float* xb = reinterpret_cast<float*>(smem_raw + a.xb_off) + (size_t)warp * 512 + lane;  // [warp][16][32]
   cplx<float>* turn = reinterpret_cast<cplx<float>*>(smem_raw + a.turn_off) + (size_t)(NW - 1 - warp) * 3 * (nvec + 1);
@@ -309,6 +310,7 @@ __global__ void __launch_bounds__(NT, 1) k_gs_step(const GsArgs a) {
       hs[v] = make_float2((float)p.x, (float)p.y);
     }
     __syncthreads();
+    if (idle && my_r >= 0 && c0 + GS_CHUNK >= nvec) givens_turn(a, my_r, turn, lane);
     for (int t = t0; t < ntiles; t += tstep) {
       const int q = 32 * t + lane;
       if (q >= a.per_g) continue;
@@ -371,7 +373,7 @@ __global__ void __launch_bounds__(NT, 1) k_gs_step(const GsArgs a) {
     s = warp_sum(s);
     if (lane == 0) __stcg(a.npart + (size_t)r * G + blockIdx.x, s);
   }
-  if (nvec > 0 && my_r >= 0) givens_turn(a, my_r, turn, lane);  // while the other CTAs arrive
+  if (nvec > 0 && my_r >= 0 && !idle) givens_turn(a, my_r, turn, lane);  // while the other CTAs arrive
   if (!grid_barrier(a.bar + 2, a.err, &ok_sh)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) a.bar[0] = a.bar[1] = 0;  // every CTA has passed them
   // ---- C: norms, the next basis vector, the Givens update
