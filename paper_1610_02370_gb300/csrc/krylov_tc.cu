@@ -558,6 +558,35 @@ __global__ void k_img_order(float* __restrict__ img, float2* __restrict__ v, int
   }
 }
 
+// canonical FP64 vectors <-> image order: one thread per complex entry of a site's vector, blockIdx.y takes every
+// gridDim.y-th right-hand side; canonical memory in order, runs of 8 entries in image order
+__device__ __forceinline__ size_t img_entry(int r, int q, int n, int b_half, int g_half) {
+  const int s = q / n, k = q - s * n;
+  return (size_t)s * b_half + (size_t)(r >> 2) * g_half + (k >> 3) * 64 + (r & 3) * 16 + (k & 7);
+}
+__global__ void k_img_from_canon(__half* __restrict__ image, float* __restrict__ img, const double2* __restrict__ x, int nc,
+                                 int n, int b_half, int g_half, int R) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= nc) return;
+  for (int r = blockIdx.y; r < R; r += gridDim.y) {
+    const double2 z = __ldg(x + (size_t)r * nc + q);
+    const float re = (float)z.x, im = (float)z.y;
+    const size_t o = img_entry(r, q, n, b_half, g_half);
+    img[o] = re;
+    img[o + 8] = im;
+    image[o] = __float2half_rn(re);
+    image[o + 8] = __float2half_rn(im);
+  }
+}
+__global__ void k_img_to_canon(double2* __restrict__ y, const float* __restrict__ img, int nc, int n, int b_half, int g_half, int R) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= nc) return;
+  for (int r = blockIdx.y; r < R; r += gridDim.y) {
+    const size_t o = img_entry(r, q, n, b_half, g_half);
+    y[(size_t)r * nc + q] = make_double2((double)img[o], (double)img[o + 8]);
+  }
+}
+
 __global__ void k_img_half(uint4* __restrict__ out, const float4* __restrict__ in, size_t n8) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n8) return;
@@ -592,6 +621,24 @@ void launch_img_order(const ImgVec& v, float* img, cplx<float>* inter, int dir, 
   k_img_order<<<(unsigned)((items + 127) / 128), 128, 0, st>>>(img, reinterpret_cast<float2*>(inter), v.t.R, v.t.n, v.t.ngj,
                                                                kg4, v.t.b_bytes / 2, v.t.sbo / 2, items, dir);
   CKL("img_order");
+}
+void launch_img_from_canon(const ImgVec& v, void* image, float* img, const double* x, cudaStream_t st) {
+  ScopedTimer timer_("img_order", st, v.t.R);
+  const int nc = v.nsites * v.t.n;
+  if (v.t.n != v.t.kpad || v.t.R % 4) {  // padding entries
+    CK(cudaMemsetAsync(image, 0, v.entries() * sizeof(__half), st));
+    CK(cudaMemsetAsync(img, 0, v.entries() * sizeof(float), st));
+  }
+  k_img_from_canon<<<dim3((nc + 255) / 256, v.t.R < 65535 ? v.t.R : 65535), 256, 0, st>>>(
+      (__half*)image, img, (const double2*)x, nc, v.t.n, v.t.b_bytes / 2, v.t.sbo / 2, v.t.R);
+  CKL("img_from_canon");
+}
+void launch_img_to_canon(const ImgVec& v, double* y, const float* img, cudaStream_t st) {
+  ScopedTimer timer_("img_order", st, v.t.R);
+  const int nc = v.nsites * v.t.n;
+  k_img_to_canon<<<dim3((nc + 255) / 256, v.t.R < 65535 ? v.t.R : 65535), 256, 0, st>>>((double2*)y, img, nc, v.t.n,
+                                                                                       v.t.b_bytes / 2, v.t.sbo / 2, v.t.R);
+  CKL("img_to_canon");
 }
 void launch_img_half(const ImgVec& v, void* out, const float* in, cudaStream_t st) {
   const size_t n8 = v.entries() / 8;

@@ -39,6 +39,10 @@ void launch_gs_step(const ImgVec& v, const void* V, size_t ldv, int nvec, float*
 void launch_img_combine(const ImgVec& v, float* x, const void* V, size_t ldv, int nvec, const double2* y, cudaStream_t st);
 // interleaved FP32 batch (element (e, r) at e R + r) <-> image-ordered FP32 (dir 0: in, 1: out)
 void launch_img_order(const ImgVec& v, float* img, cplx<float>* inter, int dir, cudaStream_t st);
+// R canonical FP64 vectors (x[r][site n + k]) -> FP16 image and image-ordered FP32 batch
+void launch_img_from_canon(const ImgVec& v, void* image, float* img, const double* x, cudaStream_t st);
+// image-ordered FP32 batch -> canonical FP64 vectors
+void launch_img_to_canon(const ImgVec& v, double* y, const float* img, cudaStream_t st);
 // FP16 image of an image-ordered FP32 batch
 void launch_img_half(const ImgVec& v, void* out, const float* in, cudaStream_t st);
 // w = b - w

@@ -1036,6 +1036,19 @@ static void coarse_out(ddtm_ctx* c, const CoarseLevel& L, double* x, cplx<float>
     unstage_out(c, x + 2 * nc * r, dout, nc, loc);
   }
 }
+// D_c(mu) on the image xt of full-lattice vectors
+static TcPass full_pass(const CoarseLevel& L, const void* xt, double mu) {
+  TcPass f;
+  f.name = "coarse_tc_full";
+  f.self = f.hops = true;
+  f.A_self = f.A_hop = L.Dct.p;
+  f.a_self_stride = 9 * (size_t)tc_geom(L.n, 1).a_bytes;
+  f.X_self = f.X_hop = xt;
+  f.tab = L.nbr.as<int>();
+  f.nout = L.Nc;
+  f.mu_c = (float)mu;
+  return f;
+}
 static CoarseLevel& level_op(ddtm_ctx* c, int level) { return level == 2 ? c->c2 : c->c1; }
 static void check_tc_all(ddtm_ctx* c) {
   check_tc_error(c->c1);
@@ -1305,6 +1318,26 @@ int ddtm_apply_Dc(ddtm_ctx* ctx, int level, double* y, const double* x, int nrhs
   if (nrhs == 0) return DDTM_OK;
   CoarseLevel& L = level_op(ctx, level);
   const size_t nc = (size_t)L.Nc * L.n;
+  const bool apart = y + 2 * nc * nrhs <= x || x + 2 * nc * nrhs <= y;
+  if (L.prec == PREC_F16 && loc == DDTM_LOC_DEVICE && apart) {
+    // canonical vectors to operand images and back in one launch each, image-ordered FP32 between (12 vectors of
+    // 32^3 x 64: 56 us for both, through interleaved batches 72 and a batch more in memory)
+    const ImgVec v{tc_geom(L.n, nrhs), L.Nc};
+    char* xt = (char*)ctx->scratch.get("abi_ct", tc_vector_image_bytes(L, L.Nc, nrhs));
+    float* xi = (float*)ctx->scratch.get("abi_ci", v.entries() * sizeof(float));
+    float* yi = (float*)ctx->scratch.get("abi_cib", v.entries() * sizeof(float));
+    launch_img_from_canon(v, xt, xi, x, ctx->stream);
+    TcPass f = full_pass(L, xt, mu);
+    f.y = reinterpret_cast<cplx<float>*>(yi);
+    f.y_img = true;
+    f.xs = xi;
+    f.xs_type = 4;
+    launch_coarse_tc(L, f, nrhs, ctx->stream);
+    launch_img_to_canon(v, y, yi, ctx->stream);
+    CK(cudaStreamSynchronize(ctx->stream));
+    check_tc_error(L);
+    return DDTM_OK;
+  }
   // all right-hand sides go through one batched stencil pass
   cplx<float>* xv = (cplx<float>*)ctx->scratch.get("abi_c32", nc * nrhs * 8);
   cplx<float>* yv = (cplx<float>*)ctx->scratch.get("abi_c32b", nc * nrhs * 8);
@@ -1312,17 +1345,9 @@ int ddtm_apply_Dc(ddtm_ctx* ctx, int level, double* y, const double* x, int nrhs
   if (L.prec == PREC_F16) {
     char* xt = (char*)ctx->scratch.get("abi_ct", tc_vector_image_bytes(L, L.Nc, nrhs));
     launch_vector_image(L, xt, xv, 1, L.Nc, nrhs, ctx->stream);
-    TcPass f;
-    f.name = "coarse_tc_full";
-    f.self = f.hops = true;
-    f.A_self = f.A_hop = L.Dct.p;
-    f.a_self_stride = 9 * (size_t)tc_geom(L.n, 1).a_bytes;
-    f.X_self = f.X_hop = xt;
-    f.tab = L.nbr.as<int>();
-    f.nout = L.Nc;
+    TcPass f = full_pass(L, xt, mu);
     f.y = yv;
     f.xs = xv;
-    f.mu_c = (float)mu;
     launch_coarse_tc(L, f, nrhs, ctx->stream);
   } else {
     launch_coarse_apply_full(L, yv, xv, nrhs, mu, 3, 1.f, 0.f, ctx->stream);

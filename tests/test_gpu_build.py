@@ -52,3 +52,28 @@ def test_aggregation_and_galerkin(lib, dims, block, nv):
             assert relerr(y[r].cpu().numpy(), cop.apply(x[r].numpy(), 0.02)) < 2e-3
     finally:
         lib.ddtm_destroy(ctx)
+
+
+@pytest.mark.parametrize("nv,nrhs", [(24, 1), (21, 5), (9, 40)])
+def test_coarse_apply_in_place_and_host(lib, nv, nrhs):
+    """D_c x from device arrays (straight between canonical vectors and operand images), in place and from host arrays
+    (through the interleaved batch) is the same, bit for bit."""
+    dims = (8, 8, 8, 16)
+    U = synth.gauge_field(dims, 0.3, seed=44).cuda()
+    ctx = lib.ddtm_create(dims, (4, 4, 4, 4), 0)
+    try:
+        lib.ddtm_load_gauge(ctx, U, 0.13, 1.2)
+        p = lib.ddtm_get_params(ctx)
+        p.nv[0], p.coarse_prec = nv, lib.PREC_F16
+        lib.ddtm_set_params(ctx, p)
+        lib.ddtm_set_test_vectors(ctx, 0, synth.gaussian_vectors((nv, 8, 16, 8, 8, 4, 3), seed=45).cuda(), nv)
+        x = synth.gaussian_vectors((nrhs, 2, 4, 2, 2, 2 * nv), seed=46)
+        y = torch.zeros_like(x).cuda()
+        lib.ddtm_apply_Dc(ctx, 1, y, x.cuda(), nrhs, 0.03)
+        z = x.cuda()
+        lib.ddtm_apply_Dc(ctx, 1, z, z, nrhs, 0.03)
+        h = torch.zeros_like(x)
+        lib.ddtm_apply_Dc(ctx, 1, h, x, nrhs, 0.03)
+        assert torch.equal(y, z) and torch.equal(y.cpu(), h)
+    finally:
+        lib.ddtm_destroy(ctx)
