@@ -179,6 +179,33 @@ __global__ void __launch_bounds__(256) k_bdots_sep(const TV* __restrict__ V, siz
   }
 }
 
+// |w(., r)|^2 of separate sets: partial[r G + CTA].  Four chains of fused multiply-adds per thread; the general inner
+// product forms the imaginary part too, and each product costs a multiplication and two additions:
+// 12 FP64 vectors of 24^3 x 48 take about 0.25 ms (DRAM) instead of 4.1.
+template <typename T>
+__global__ void __launch_bounds__(256) k_bnorm_sep(const T* __restrict__ w, size_t n, double2* __restrict__ partial) {
+  __shared__ double red[16];
+  const int G = gridDim.x, r = blockIdx.y;
+  const T* a = w + (size_t)r * n;
+  typedef typename Acc<T, T>::T AT;
+  AT s[4] = {0, 0, 0, 0};
+  const size_t step = (size_t)G * 256;
+  size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  for (; i + 3 * step < n; i += 4 * step) {
+    cplx<AT> v[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) v[u] = ldc<AT>(a, i + u * step);
+#pragma unroll
+    for (int u = 0; u < 4; u++) s[u] = fma(v[u].re, v[u].re, fma(v[u].im, v[u].im, s[u]));
+  }
+  for (; i < n; i += step) {
+    const cplx<AT> v = ldc<AT>(a, i);
+    s[0] = fma(v.re, v.re, fma(v.im, v.im, s[0]));
+  }
+  const double2 t = cta_reduce(make_double2(((double)s[0] + (double)s[1]) + ((double)s[2] + (double)s[3]), 0), red);
+  if (threadIdx.x == 0) partial[(size_t)r * G + blockIdx.x] = t;
+}
+
 // Interleaved FP32 sets with an even number R of right-hand sides, read in
 // 16-byte pairs (two consecutive right-hand sides of one entry).  Work comes
 // in spans of EPT x blockDim consecutive pairs: thread t of a CTA takes pairs
@@ -403,6 +430,131 @@ __global__ void k_bmaxpy(TW* __restrict__ w, const TV* __restrict__ V, size_t ld
     if (npartial) {
       double2 s = cta_reduce(make_double2((double)nn, 0), reinterpret_cast<double*>(red));
       if (threadIdx.x == 0) npartial[(size_t)r_sep * G + blockIdx.x] = s;
+    }
+  }
+}
+
+// ---- Gram-Schmidt of separate FP32 vectors (the outer Arnoldi process) ----------------------------------------
+// One sweep over w in tiles of GF_TILE pairs (two complex entries, 16 bytes), a tile of w in registers:
+//   SUB   w -= sum_j coef[j R + r] V_j, and w is stored
+//   NORM  npartial[r G + CTA] = |w|^2 of the CTA's tiles
+//   DOT   partial[(j R + r) G + CTA] = <V_j, w> of the CTA's tiles, w as it is after SUB
+// SUB + DOT is the end of the first projection and the inner products of the second in one pass: the tile's basis
+// entries are read twice, in descending order the second time, so that they come from L1 and L2.  CTA (c, r) takes
+// tiles c, c + G, ... of right-hand side r.  A lane sums eight products per tile and vector, the warp sums by shuffles
+// in FP32, and lane j adds the tile's result for vector j in FP64: one FP64 addition per 32 vectors and warp.
+// Bound by DRAM.  12 right-hand sides of 24^3 x 48, 6.5 vectors on average: inner products 0.81 ms (6.7 TB/s of its
+// bytes; before 1.02), SUB + DOT 1.32 ms (5.1 TB/s; the second reading misses L2 in part), SUB + NORM 1.16 ms (5.8);
+// two projections 3.3 ms, with one launch per product and update 5.1.
+static const int GF_THREADS = 256, GF_EPT = 2, GF_TILE = GF_THREADS * GF_EPT, GF_U = 4;
+template <bool SUB, bool NORM, bool DOT>
+__global__ void __launch_bounds__(GF_THREADS, 2) k_gs_fine(float4* __restrict__ w, const float4* __restrict__ V, size_t ldv,
+                                                           int nvec, const double2* __restrict__ coef, size_t n2, int R,
+                                                           double2* __restrict__ partial, double2* __restrict__ npartial) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[2 * GF_THREADS / 32];
+  constexpr int NW = GF_THREADS / 32;
+  const int G = gridDim.x, r = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  double2* acc = reinterpret_cast<double2*>(smem_raw);                                // DOT: [NW][nvec]
+  float2* hc = reinterpret_cast<float2*>(smem_raw + (DOT ? (size_t)NW * nvec * sizeof(double2) : 0));  // SUB: [nvec]
+  if (SUB)
+    for (int j = t; j < nvec; j += GF_THREADS) {
+      const double2 c = coef[(size_t)j * R + r];
+      hc[j] = make_float2((float)c.x, (float)c.y);
+    }
+  if (DOT)
+    for (int j = t; j < NW * nvec; j += GF_THREADS) acc[j] = make_double2(0, 0);
+  __syncthreads();
+  float4* wr = w + (size_t)r * n2;
+  const float4* Vr = V + (size_t)r * n2;
+  double nn = 0;
+  for (size_t base = (size_t)blockIdx.x * GF_TILE; base < n2; base += (size_t)G * GF_TILE) {
+    size_t i[GF_EPT];
+    bool in[GF_EPT];
+    float4 x[GF_EPT];
+#pragma unroll
+    for (int e = 0; e < GF_EPT; e++) {
+      i[e] = base + t + (size_t)e * GF_THREADS;
+      in[e] = i[e] < n2;
+      if (!in[e]) i[e] = n2 - 1;  // an entry of the vector, with zero weight below
+      x[e] = in[e] ? wr[i[e]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (SUB) {
+      for (int j0 = 0; j0 < nvec; j0 += GF_U) {
+        float4 v[GF_U][GF_EPT];
+#pragma unroll
+        for (int u = 0; u < GF_U; u++)
+#pragma unroll
+          for (int e = 0; e < GF_EPT; e++) v[u][e] = __ldg(Vr + (size_t)(j0 + u < nvec ? j0 + u : nvec - 1) * ldv + i[e]);
+#pragma unroll
+        for (int u = 0; u < GF_U; u++) {
+          if (j0 + u >= nvec) break;
+          const float2 h = hc[j0 + u];
+#pragma unroll
+          for (int e = 0; e < GF_EPT; e++) {
+            x[e].x -= h.x * v[u][e].x - h.y * v[u][e].y;
+            x[e].y -= h.x * v[u][e].y + h.y * v[u][e].x;
+            x[e].z -= h.x * v[u][e].z - h.y * v[u][e].w;
+            x[e].w -= h.x * v[u][e].w + h.y * v[u][e].z;
+          }
+        }
+      }
+      float s = 0.f;
+#pragma unroll
+      for (int e = 0; e < GF_EPT; e++) {
+        if (in[e]) wr[i[e]] = x[e];
+        else x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        s += x[e].x * x[e].x + x[e].y * x[e].y + x[e].z * x[e].z + x[e].w * x[e].w;
+      }
+      if (NORM) nn += (double)s;
+    }
+    if (DOT)
+      for (int c0 = (nvec - 1) & ~31; c0 >= 0; c0 -= 32) {
+        const int top = nvec - c0 < 32 ? nvec : c0 + 32;
+        float pr = 0.f, pi = 0.f;
+        for (int j0 = top - 1; j0 >= c0; j0 -= GF_U) {
+          float4 v[GF_U][GF_EPT];
+#pragma unroll
+          for (int u = 0; u < GF_U; u++)
+#pragma unroll
+            for (int e = 0; e < GF_EPT; e++) v[u][e] = __ldg(Vr + (size_t)(j0 - u >= c0 ? j0 - u : c0) * ldv + i[e]);
+#pragma unroll
+          for (int u = 0; u < GF_U; u++) {
+            float sr = 0.f, si = 0.f;
+#pragma unroll
+            for (int e = 0; e < GF_EPT; e++) {
+              const float4 a = v[u][e], b = x[e];
+              sr += a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w;
+              si += a.x * b.y - a.y * b.x + a.z * b.w - a.w * b.z;
+            }
+            sr = warp_sum(sr);
+            si = warp_sum(si);
+            if (lane == j0 - u - c0) {
+              pr = sr;
+              pi = si;
+            }
+          }
+        }
+        if (c0 + lane < top) {
+          double2* p = acc + (size_t)warp * nvec + c0 + lane;
+          p->x += (double)pr;
+          p->y += (double)pi;
+        }
+      }
+  }
+  if (NORM) {
+    const double2 s = cta_reduce(make_double2(nn, 0), red);
+    if (t == 0) npartial[(size_t)r * G + blockIdx.x] = s;
+  }
+  if (DOT) {
+    __syncthreads();
+    for (int j = t; j < nvec; j += GF_THREADS) {
+      double2 s = acc[j];
+      for (int k = 1; k < NW; k++) {
+        s.x += acc[(size_t)k * nvec + j].x;
+        s.y += acc[(size_t)k * nvec + j].y;
+      }
+      partial[((size_t)j * R + r) * G + blockIdx.x] = s;
     }
   }
 }
@@ -712,7 +864,10 @@ void Blas::dots(const VSet& V, size_t ldv, int nvec, const VSet& w, double2* out
   else if (w.inter)
     DISPATCH_TYPES(V.type, w.type,
                    (k_bdots<A, B, true><<<grid, bd, 0, st>>>((const A*)V.p, ldv, nvec, (const B*)w.p, w.n, R, partial)));
-  else
+  else if (V.p == w.p && nvec == 1 && V.type == w.type && w.type != 2) {
+    if (w.type == 0) k_bnorm_sep<double2><<<dim3(G, R), 256, 0, st>>>((const double2*)w.p, w.n, partial);
+    else k_bnorm_sep<float2><<<dim3(G, R), 256, 0, st>>>((const float2*)w.p, w.n, partial);
+  } else
     DISPATCH_TYPES(V.type, w.type,
                    (k_bdots_sep<A, B, SEP_JB><<<dim3(G, (nvec + SEP_JB - 1) / SEP_JB, R), bd, 0, st>>>(
                        (const A*)V.p, ldv, nvec, (const B*)w.p, w.n, R, partial)));
@@ -862,6 +1017,50 @@ void Blas::maxpy_dev(const VSet& w, const VSet& V, size_t ldv, int nvec, const d
     k_reduce_partials<<<R, 128, 0, st>>>(npart, G, norms2_dev);
     CKL("reduce_partials");
   }
+}
+
+static size_t gs_fine_smem(bool sub, bool dot, int nvec) {
+  return (size_t)nvec * ((dot ? GF_THREADS / 32 * sizeof(double2) : 0) + (sub ? sizeof(float2) : 0));
+}
+template <bool SUB, bool NORM, bool DOT>
+static void gs_fine(Blas* b, const VSet& w, const VSet& V, size_t ldv, int nvec, const double2* coef, double2* out) {
+  const size_t n2 = w.n / 2, tiles = (n2 + GF_TILE - 1) / GF_TILE, smem = gs_fine_smem(SUB, DOT, nvec);
+  auto kernel = k_gs_fine<SUB, NORM, DOT>;
+  set_dynamic_smem((const void*)kernel, 200 * 1024);
+  const int G = span_grid(tiles, w.R, resident_ctas((const void*)kernel, GF_THREADS, smem));
+  const int rows = DOT ? nvec * w.R : w.R;
+  double2* part = (double2*)b->pool->get("blas_gs_partial", (size_t)rows * G * sizeof(double2));
+  kernel<<<dim3(G, w.R), GF_THREADS, smem, b->st>>>((float4*)w.p, (const float4*)V.p, ldv / 2, nvec, coef, n2, w.R, part, part);
+  CKL("gs_fine");
+  k_reduce_partials<<<rows, 128, 0, b->st>>>(part, G, out);
+  CKL("reduce_partials");
+}
+
+// Two projections cost three sweeps of the basis for separate FP32 vectors (k_gs_fine: FP32, an even number of entries,
+// 16-byte addresses; every outer vector of 12 V entries has them), four otherwise (FP64 cycles, whose arithmetic is bound
+// by the FP64 units, and bases whose coefficients exceed the shared-memory stage).
+void Blas::gram_schmidt2_dev(const VSet& w, const VSet& V, size_t ldv, int nvec, double2* h, double2* h2, double2* norms2_dev) {
+  const bool fine = !w.inter && !V.inter && w.type == 1 && V.type == 1 && w.n && w.n % 2 == 0 && ldv % 2 == 0 && nvec > 0 &&
+                    w.R <= 65535 && ((uintptr_t)V.p & 15) == 0 && ((uintptr_t)w.p & 15) == 0 &&
+                    gs_fine_smem(true, true, nvec) <= 96 * 1024;
+  if (!fine) {
+    dots_dev(V, ldv, nvec, w, h);
+    maxpy_dev(w, V, ldv, nvec, h, -1.0, nullptr);
+    dots_dev(V, ldv, nvec, w, h2);
+    maxpy_dev(w, V, ldv, nvec, h2, -1.0, norms2_dev);
+    return;
+  }
+  const double vb = nvec * set_bytes(V), wb = set_bytes(w);
+  {
+    ScopedTimer timer_("blas_dots_fine", st, nvec, vb + wb);
+    gs_fine<false, false, true>(this, w, V, ldv, nvec, nullptr, h);
+  }
+  {
+    ScopedTimer timer_("blas_maxpy_dots_fine", st, 2 * nvec, vb + 2 * wb);
+    gs_fine<true, false, true>(this, w, V, ldv, nvec, h, h2);
+  }
+  ScopedTimer timer_("blas_maxpy_fine", st, nvec, vb + 2 * wb);
+  gs_fine<true, true, false>(this, w, V, ldv, nvec, h2, norms2_dev);
 }
 
 void Blas::scale_dev(const double2* a_dev, const VSet& x, const VSet& y) {

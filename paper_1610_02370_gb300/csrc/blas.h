@@ -50,6 +50,8 @@ struct Blas {
   void dots_dev(const VSet& V, size_t ldv, int nvec, const VSet& w, double2* out_dev);
   void maxpy_dev(const VSet& w, const VSet& V, size_t ldv, int nvec, const double2* coef_dev, double sign,
                  double2* norms2_dev);
+  // classical Gram-Schmidt, twice: h = V^+ w, w -= V h, h2 = V^+ w, w -= V h2 and ||w||^2
+  void gram_schmidt2_dev(const VSet& w, const VSet& V, size_t ldv, int nvec, double2* h, double2* h2, double2* norms2_dev);
   // y(., r) = a[r] x(., r), a in device memory
   void scale_dev(const double2* a_dev, const VSet& x, const VSet& y);
 

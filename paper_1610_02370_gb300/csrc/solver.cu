@@ -853,10 +853,7 @@ OuterResult outer_fgmres(ddtm_ctx* c, double* x, const double* b, double mu, int
         zin = t32;
       }
       Dcyc(w, zin);
-      B.dots_dev(sc_(V), (size_t)R * n, j + 1, sc_(w), h);
-      B.maxpy_dev(sc_(w), sc_(V), (size_t)R * n, j + 1, h, -1.0, nullptr);
-      B.dots_dev(sc_(V), (size_t)R * n, j + 1, sc_(w), h2);
-      B.maxpy_dev(sc_(w), sc_(V), (size_t)R * n, j + 1, h2, -1.0, nr2);
+      B.gram_schmidt2_dev(sc_(w), sc_(V), (size_t)R * n, j + 1, h, h2, nr2);
       launch_arnoldi_step(ad, j, h, h2, nr2, c->stream, false);
       fetch_est(j & 1);
       if (j < m - 1) B.scale_dev(ad.scale, sc_(w), sc_(Vj(j + 1)));
