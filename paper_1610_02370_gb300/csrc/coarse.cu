@@ -595,114 +595,137 @@ __device__ __forceinline__ void block_mv2(const DS* A, const cplx<float>* v, int
   }
 }
 
-// Threads of a site: n/2 row pairs x G chunk slots, row pair fastest (a warp
-// reads consecutive 16-byte pieces of a column); a thread takes the chunks
-// ch = g, g + G, ... of RC right-hand sides (launch_shape.h); SPB sites per CTA.
-template <typename DS, int RC>
-__global__ void __launch_bounds__(256) k_coarse_apply(cplx<float>* __restrict__ y, const cplx<float>* __restrict__ x_self,
-                                                       const cplx<float>* __restrict__ x_hop, const DS* __restrict__ Dc,
-                                                       const int* __restrict__ tab, const int* __restrict__ osite, int nout,
-                                                       int n, int nv, int R, int G, float mu_c, int mode, float sres,
-                                                       float sy, int dsel) {
+// One hop of the stencil, y[site] = A_d(site) x[site + d].  Threads of a site: n/2 row pairs x G chunk slots, row pair
+// fastest (a warp reads consecutive 16-byte pieces of a column); a thread takes the chunks ch = g, g + G, ... of RC
+// right-hand sides (launch_shape.h); SPB sites per CTA.
+template <int RC>
+__global__ void __launch_bounds__(256) k_coarse_hop(cplx<float>* __restrict__ y, const cplx<float>* __restrict__ x,
+                                                     const float2* __restrict__ Dc, const int* __restrict__ nbr, int nout, int n,
+                                                     int R, int G, int d) {
   const int np = n / 2, nch = R / RC, per = np * G, spb = blockDim.x / per;
   const int t = threadIdx.x, rp = t % np, g = (t / np) % G, q = t / per;
-  const int idx = blockIdx.x * spb + q;
-  if (q >= spb || idx >= nout) return;
-  const int site = osite ? osite[idx] : idx;
-  const int r0 = 2 * rp;
-  for (int ch = g; ch < nch; ch += G) {
-  const int c0 = ch * RC;
-  cplx<float> acc0[RC], acc1[RC];
-#pragma unroll
-  for (int c = 0; c < RC; c++) acc0[c] = acc1[c] = cplx<float>(0, 0);
-  if (mode & 1) {
-    block_mv2<DS, RC>(Dc + (size_t)site * 9 * n * n + r0, x_self + (size_t)idx * n * R + c0, n, R, acc0, acc1);
-    cplx<float> xv0[RC], xv1[RC];
-    load_rc<RC>(x_self + ((size_t)idx * n + r0) * R + c0, xv0);
-    load_rc<RC>(x_self + ((size_t)idx * n + r0 + 1) * R + c0, xv1);
-    const float m0 = r0 < nv ? mu_c : -mu_c, m1 = r0 + 1 < nv ? mu_c : -mu_c;
-#pragma unroll
-    for (int c = 0; c < RC; c++) {
-      acc0[c] = acc0[c] + m0 * times_i(xv0[c]);
-      acc1[c] = acc1[c] + m1 * times_i(xv1[c]);
-    }
-  }
-  if (mode & 2)
-    for (int d = dsel ? dsel : 1; d <= (dsel ? dsel : 8); d++) {  // dsel > 0: hop dsel - 1 only
-      const int src = __ldg(tab + (size_t)(d - 1) * nout + idx);
-      block_mv2<DS, RC>(Dc + ((size_t)site * 9 + d) * n * n + r0, x_hop + (size_t)src * n * R + c0, n, R, acc0, acc1);
-    }
-  cplx<float>* yo0 = y + ((size_t)idx * n + r0) * R + c0;
-  cplx<float>* yo1 = yo0 + R;
-#pragma unroll
-  for (int c = 0; c < RC; c++) {
-    cplx<float> res0 = sres * acc0[c], res1 = sres * acc1[c];
-    yo0[c] = sy == 0.f ? res0 : sy * yo0[c] + res0;
-    yo1[c] = sy == 0.f ? res1 : sy * yo1[c] + res1;
-  }
-  }
-}
-
-// t[e] = Dinv_e (sr * rhs[e] + sh * hops(v)) on the even sites (compact even
-// output, v compact odd); rhs or v may be null.  Hop and inverse are fused:
-// the hop result of a site goes through shared memory to the threads of the
-// same site for the dense matvec with the inverse.
-template <typename DS, int RC>
-__global__ void __launch_bounds__(256) k_coarse_even(cplx<float>* __restrict__ t, const cplx<float>* __restrict__ rhs,
-                                                      const cplx<float>* __restrict__ v, const DS* __restrict__ Dc,
-                                                      const float2* __restrict__ Dinv, const int* __restrict__ tab,
-                                                      const int* __restrict__ even, int ne, int n, int R, int G, float sr,
-                                                      float sh) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int np = n / 2, nch = R / RC, per = np * G, spb = blockDim.x / per;
-  cplx<float>* hs = reinterpret_cast<cplx<float>*>(smem_raw);  // [spb][n][R]
-  const int th = threadIdx.x, rp = th % np, g = (th / np) % G, q = th / per;
-  const int e = blockIdx.x * spb + q;
-  const bool act = q < spb && e < ne;
-  const int r0 = 2 * rp;
-  if (act)
+  const int site = blockIdx.x * spb + q;
+  if (q >= spb || site >= nout) return;
+  const int r0 = 2 * rp, src = __ldg(nbr + (size_t)(d - 1) * nout + site);
   for (int ch = g; ch < nch; ch += G) {
     const int c0 = ch * RC;
-    const int site = even[e];
     cplx<float> acc0[RC], acc1[RC];
 #pragma unroll
     for (int c = 0; c < RC; c++) acc0[c] = acc1[c] = cplx<float>(0, 0);
-    if (v)
-      for (int d = 1; d < 9; d++) {
-        const int src = __ldg(tab + (size_t)(d - 1) * ne + e);
-        block_mv2<DS, RC>(Dc + ((size_t)site * 9 + d) * n * n + r0, v + (size_t)src * n * R + c0, n, R, acc0, acc1);
-      }
-    cplx<float> rv0[RC], rv1[RC];
-    if (rhs) {
-      load_rc<RC>(rhs + ((size_t)e * n + r0) * R + c0, rv0);
-      load_rc<RC>(rhs + ((size_t)e * n + r0 + 1) * R + c0, rv1);
-    }
+    block_mv2<float2, RC>(Dc + ((size_t)site * 9 + d) * n * n + r0, x + (size_t)src * n * R + c0, n, R, acc0, acc1);
+    cplx<float>* yo = y + ((size_t)site * n + r0) * R + c0;
 #pragma unroll
     for (int c = 0; c < RC; c++) {
-      cplx<float> a0 = sh * acc0[c], a1 = sh * acc1[c];
-      if (rhs) {
-        a0 = a0 + sr * rv0[c];
-        a1 = a1 + sr * rv1[c];
-      }
-      hs[((size_t)q * n + r0) * R + c0 + c] = a0;
-      hs[((size_t)q * n + r0 + 1) * R + c0 + c] = a1;
+      yo[c] = acc0[c];
+      yo[R + c] = acc1[c];
     }
   }
-  __syncthreads();
-  if (act)
-  for (int ch = g; ch < nch; ch += G) {
-    const int c0 = ch * RC;
-    cplx<float> o0[RC], o1[RC];
+}
+
+// The stencil with a CTA per site and chunk of RC right-hand sides: n/2 row pairs x S shares of the products.  Unit
+// u = d H + h is part h of H (columns h n / H ...) of hop d (d = 0: the self block); share s takes units s, s + S, ...,
+// and every unit's result goes to shared memory, where the units are summed in order: the result depends neither on S
+// nor on the batch.  With an inverse (even sites, Dinv != null) the sum hs = sr rhs + sres (hops) is multiplied by it,
+// the columns shared out in the same way.  The last chunk may have fewer columns than RC.
+// One thread per row pair for all of the hops, as for single hops (k_coarse_hop), is a chain of 9 n loads of 16 bytes and leaves most SMs
+// without work on coarse lattices of a few hundred sites.  Full stencil in FP32, before ->
+// after, 48 dofs: 32 sites, 1 column 65 -> 10 us, 12 columns 70 -> 14; 512 sites 76 -> 24, 113 to 165 -> 86; 2592 sites
+// 194 -> 129, 352 -> 350.  Bound by the matrices (430 MB at 2592 sites) with one column and by shared loads of the
+// vectors' columns with many.
+// COLS: 0 all RC columns are there, 1 nc <= RC of them (any R), 2 the same with an even R
+template <int RC, int COLS>
+__device__ __forceinline__ void load_cols(const cplx<float>* p, int nc, cplx<float> v[RC]) {
+  if (COLS == 0) {
+    load_rc<RC>(p, v);
+  } else if (COLS == 1) {
 #pragma unroll
-    for (int c = 0; c < RC; c++) o0[c] = o1[c] = cplx<float>(0, 0);
-    block_mv2<float2, RC>(Dinv + (size_t)e * n * n + r0, hs + (size_t)q * n * R + c0, n, R, o0, o1);
-    cplx<float>* to0 = t + ((size_t)e * n + r0) * R + c0;
-    cplx<float>* to1 = to0 + R;
+    for (int c = 0; c < RC; c++) v[c] = c < nc ? p[c] : cplx<float>(0, 0);
+  } else {
+#pragma unroll
+    for (int c = 0; c + 1 < RC; c += 2) {
+      const float4 a = c < nc ? *reinterpret_cast<const float4*>(p + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[c] = cplx<float>(a.x, a.y);
+      v[c + 1] = cplx<float>(a.z, a.w);
+    }
+  }
+}
+// part[row][c] = sum_k A[row][k] x[k][c] of the rows r0, r0 + 1 (x rows R apart) for kn columns
+template <int RC, int COLS>
+__device__ __forceinline__ void split_unit(cplx<float>* part, const float2* A, const cplx<float>* x, int n, int kn, int R, int nc) {
+  cplx<float> acc0[RC], acc1[RC];
+#pragma unroll
+  for (int c = 0; c < RC; c++) acc0[c] = acc1[c] = cplx<float>(0, 0);
+#pragma unroll 8
+  for (int k = 0; k < kn; k++) {
+    cplx<float> a0, a1, v[RC];
+    ld_rows2<float2>(A + (size_t)k * n, a0, a1);
+    load_cols<RC, COLS>(x + (size_t)k * R, nc, v);
 #pragma unroll
     for (int c = 0; c < RC; c++) {
-      to0[c] = o0[c];
-      to1[c] = o1[c];
+      cmac(acc0[c], a0, v[c]);
+      cmac(acc1[c], a1, v[c]);
     }
+  }
+#pragma unroll
+  for (int c = 0; c < RC; c++) {
+    part[c] = acc0[c];
+    part[RC + c] = acc1[c];
+  }
+}
+__device__ __forceinline__ cplx<float> split_sum(const cplx<float>* part, int units, int nrc, int k) {
+  cplx<float> v = part[k];
+  for (int u = 1; u < units; u++) v = v + part[(size_t)u * nrc + k];
+  return v;
+}
+static const int SPLIT_KU = 8;  // shares of the inverse's columns
+template <int RC, int COLS>
+__global__ void __launch_bounds__(1024)
+    k_coarse_split(cplx<float>* __restrict__ y, const cplx<float>* __restrict__ x_self, const cplx<float>* __restrict__ x_hop,
+                   const float2* __restrict__ Dc, const int* __restrict__ tab, const int* __restrict__ osite, int nout, int n,
+                   int nv, int R, int S, int H, float mu_c, int mode, float sres, float sy, const float2* __restrict__ Dinv,
+                   const cplx<float>* __restrict__ rhs, float sr) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int np = n / 2, nch = (R + RC - 1) / RC, nrc = n * RC;
+  const int idx = blockIdx.x / nch, c0 = (blockIdx.x - idx * nch) * RC, nc = R - c0 < RC ? R - c0 : RC;
+  const int t = threadIdx.x, rp = t % np, s = t / np, r0 = 2 * rp;
+  const int site = osite ? osite[idx] : idx;
+  const int d0 = mode & 1 ? 0 : 1, d1 = mode & 2 ? 9 : 1;  // hops d0 ... d1 - 1
+  const int units = (d1 - d0) * H, kh = (n + H - 1) / H;
+  cplx<float>* part = reinterpret_cast<cplx<float>*>(smem_raw);  // [9 H][n][RC]
+  cplx<float>* hs = part + (size_t)9 * H * nrc;                  // [n][RC], with an inverse
+  for (int u = s; u < units; u += S) {
+    const int d = d0 + u / H, k0 = (u % H) * kh, kn = n - k0 < kh ? n - k0 : kh;
+    const cplx<float>* x = d ? x_hop + (size_t)__ldg(tab + (size_t)(d - 1) * nout + idx) * n * R : x_self + (size_t)idx * n * R;
+    split_unit<RC, COLS>(part + (size_t)u * nrc + (size_t)r0 * RC, Dc + (((size_t)site * 9 + d) * n + k0) * n + r0,
+                        x + (size_t)k0 * R + c0, n, kn, R, nc);
+  }
+  __syncthreads();
+  for (int k = t; k < nrc; k += blockDim.x) {
+    const int row = k / RC, c = k - row * RC;
+    const size_t o = ((size_t)idx * n + row) * R + c0 + c;
+    cplx<float> v = units > 0 ? split_sum(part, units, nrc, k) : cplx<float>(0, 0);
+    if (Dinv) {
+      v = sres * v;
+      if (rhs && c < nc) v = v + sr * rhs[o];
+      hs[k] = v;
+    } else if (c < nc) {
+      if (mode & 1) v = v + (row < nv ? mu_c : -mu_c) * times_i(x_self[o]);
+      v = sres * v;
+      y[o] = sy == 0.f ? v : sy * y[o] + v;
+    }
+  }
+  if (!Dinv) return;
+  __syncthreads();
+  const int ku = (n + SPLIT_KU - 1) / SPLIT_KU;
+  for (int u = s; u < SPLIT_KU; u += S) {
+    const int k0 = u * ku < n ? u * ku : n, kn = n - k0 < ku ? n - k0 : ku;
+    split_unit<RC, 0>(part + (size_t)u * nrc + (size_t)r0 * RC, Dinv + ((size_t)idx * n + k0) * n + r0,
+                                hs + (size_t)k0 * RC, n, kn, RC, RC);
+  }
+  __syncthreads();
+  for (int k = t; k < nrc; k += blockDim.x) {
+    const int row = k / RC, c = k - row * RC;
+    if (c < nc) y[((size_t)idx * n + row) * R + c0 + c] = split_sum(part, SPLIT_KU, nrc, k);
   }
 }
 
@@ -818,67 +841,63 @@ __global__ void k_self_inverse(float2* __restrict__ Dinv, const DS* __restrict__
     }
 }
 
-template <typename DS, int RC>
-static void coarse_apply_t(const CoarseLevel& c, const CoarseShape& sh, cplx<float>* y, const cplx<float>* xs,
-                           const cplx<float>* xh, const int* tab, const int* osite, int nout, int R, double mu_c, int mode,
-                           float sres, float sy, cudaStream_t st, int dsel) {
-  unsigned grid = (unsigned)((nout + sh.spb - 1) / sh.spb);
-  if (grid == 0) return;
-  k_coarse_apply<DS, RC><<<grid, sh.threads, 0, st>>>(y, xs, xh, c.Dc.as<DS>(), tab, osite, nout, c.n, c.nv, R, sh.groups,
-                                                      (float)mu_c, mode, sres, sy, dsel);
-  CKL("coarse_apply");
+template <int RC, int COLS>
+static void coarse_split_t(const CoarseLevel& c, cplx<float>* y, const cplx<float>* xs, const cplx<float>* xh, const int* tab,
+                           const int* osite, int nout, int R, int S, int H, size_t smem, double mu_c, int mode, float sres,
+                           float sy, const float2* Dinv, const cplx<float>* rhs, float sr, cudaStream_t st) {
+  set_dynamic_smem((const void*)k_coarse_split<RC, COLS>, 200 * 1024);
+  k_coarse_split<RC, COLS><<<(unsigned)(nout * ((R + RC - 1) / RC)), c.n / 2 * S, smem, st>>>(
+      y, xs, xh, c.Dc.as<float2>(), tab, osite, nout, c.n, c.nv, R, S, H, (float)mu_c, mode, sres, sy, Dinv, rhs, sr);
+  CKL("coarse_split");
 }
-
-template <typename DS>
-static void coarse_apply_d(const CoarseLevel& c, cplx<float>* y, const cplx<float>* xs, const cplx<float>* xh, const int* tab,
-                           const int* osite, int nout, int R, double mu_c, int mode, float sres, float sy, cudaStream_t st,
-                           int dsel = 0) {
-  const CoarseShape sh = coarse_shape(c.n, R);
-  if (sh.rc == 4) coarse_apply_t<DS, 4>(c, sh, y, xs, xh, tab, osite, nout, R, mu_c, mode, sres, sy, st, dsel);
-  else if (sh.rc == 2) coarse_apply_t<DS, 2>(c, sh, y, xs, xh, tab, osite, nout, R, mu_c, mode, sres, sy, st, dsel);
-  else coarse_apply_t<DS, 1>(c, sh, y, xs, xh, tab, osite, nout, R, mu_c, mode, sres, sy, st, dsel);
+// Units of a hop: two on lattices with at most two CTAs per SM, where the chain of a unit's loads is what counts, and one
+// beyond (2592 sites of 48 dofs, 12 columns: 350 us with one, 388 with two).  Four columns per CTA, fewer where R is 1 or
+// 2 (with 12 columns a matrix entry is loaded once for 12 right-hand sides, but the registers leave too few warps: 421).
+static void coarse_split(const CoarseLevel& c, cplx<float>* y, const cplx<float>* xs, const cplx<float>* xh, const int* tab,
+                         const int* osite, int nout, int R, double mu_c, int mode, float sres, float sy, const float2* Dinv,
+                         const cplx<float>* rhs, float sr, cudaStream_t st) {
+  if (nout == 0) return;
+  const int np = c.n / 2, H = 18 * np <= 1024 && nout <= 304 ? 2 : 1, S = std::max(1, std::min(9 * H, 1024 / np));
+  const int rc = R < 3 ? R : 4;
+  auto go = R == 1       ? coarse_split_t<1, 0>
+            : R == 2     ? coarse_split_t<2, 0>
+            : R % 4 == 0 ? coarse_split_t<4, 0>
+            : R % 2 == 0 ? coarse_split_t<4, 2>
+                         : coarse_split_t<4, 1>;
+  const size_t smem = (size_t)(9 * H + 1) * c.n * rc * sizeof(cplx<float>);  // n <= 128: at most 74 KB
+  go(c, y, xs, xh, tab, osite, nout, R, S, H, smem, mu_c, mode, sres, sy, Dinv, rhs, sr, st);
 }
 
 void launch_coarse_apply_hop(const CoarseLevel& c, cplx<float>* y, const cplx<float>* x, int R, int hop, cudaStream_t st) {
   ScopedTimer timer_("coarse_apply", st, R);
-  coarse_apply_d<float2>(c, y, x, x, c.nbr.as<int>(), nullptr, c.Nc, R, 0.0, 2, 1.f, 0.f, st, hop + 1);
+  const CoarseShape sh = coarse_shape(c.n, R);
+  const unsigned grid = (unsigned)((c.Nc + sh.spb - 1) / sh.spb);
+  auto kernel = sh.rc == 4 ? k_coarse_hop<4> : sh.rc == 2 ? k_coarse_hop<2> : k_coarse_hop<1>;
+  kernel<<<grid, sh.threads, 0, st>>>(y, x, c.Dc.as<float2>(), c.nbr.as<int>(), c.Nc, c.n, R, sh.groups, hop + 1);
+  CKL("coarse_hop");
 }
 
 void launch_coarse_apply_full(const CoarseLevel& c, cplx<float>* y, const cplx<float>* x, int R, double mu_c, int mode,
                               float sres, float sy, cudaStream_t st) {
   ScopedTimer timer_("coarse_apply", st, R);
-  coarse_apply_d<float2>(c, y, x, x, c.nbr.as<int>(), nullptr, c.Nc, R, mu_c, mode, sres, sy, st);
+  coarse_split(c, y, x, x, c.nbr.as<int>(), nullptr, c.Nc, R, mu_c, mode, sres, sy, nullptr, nullptr, 0.f, st);
 }
 
 void launch_coarse_apply_odd(const CoarseLevel& c, cplx<float>* y_o, const cplx<float>* x_o, const cplx<float>* x_e, int R,
                              double mu_c, int mode, float sres, float sy, cudaStream_t st) {
   ScopedTimer timer_("coarse_apply_odd_f32", st, R);
-  int no = (int)c.h_odd.size();
-  coarse_apply_d<float2>(c, y_o, x_o, x_e, c.nbr_oe.as<int>(), c.odd.as<int>(), no, R, mu_c, mode, sres, sy, st);
-}
-
-template <typename DS, int RC>
-static void coarse_even_t(const CoarseLevel& c, const CoarseShape& shp, cplx<float>* t, const cplx<float>* rhs,
-                          const cplx<float>* v, int R, float sr, float sh, cudaStream_t st) {
-  int ne = (int)c.h_even.size();
-  unsigned grid = (unsigned)((ne + shp.spb - 1) / shp.spb);
-  if (grid == 0) return;
-  size_t smem = (size_t)shp.spb * c.n * R * sizeof(cplx<float>);
-  if (smem > 200 * 1024) throw Error(DDTM_ERR_ARG, "coarse_even: " + std::to_string(R) + " right-hand sides of " +
-                                                       std::to_string(c.n) + " dofs exceed the shared-memory stage");
-  set_dynamic_smem((const void*)k_coarse_even<DS, RC>, 200 * 1024);
-  k_coarse_even<DS, RC><<<grid, shp.threads, smem, st>>>(t, rhs, v, c.Dc.as<DS>(), c.Dinv.as<float2>(), c.nbr_eo.as<int>(),
-                                                         c.even.as<int>(), ne, c.n, R, shp.groups, sr, sh);
-  CKL("coarse_even");
+  coarse_split(c, y_o, x_o, x_e, c.nbr_oe.as<int>(), c.odd.as<int>(), (int)c.h_odd.size(), R, mu_c, mode, sres, sy, nullptr,
+               nullptr, 0.f, st);
 }
 
 void launch_coarse_even(const CoarseLevel& c, cplx<float>* t, const cplx<float>* rhs, const cplx<float>* v, int R, float sr,
                         float sh, cudaStream_t st) {
   ScopedTimer timer_("coarse_even_f32", st, R);
-  const CoarseShape shp = coarse_shape(c.n, R);
-  if (shp.rc == 4) coarse_even_t<float2, 4>(c, shp, t, rhs, v, R, sr, sh, st);
-  else if (shp.rc == 2) coarse_even_t<float2, 2>(c, shp, t, rhs, v, R, sr, sh, st);
-  else coarse_even_t<float2, 1>(c, shp, t, rhs, v, R, sr, sh, st);
+  if ((size_t)coarse_shape(c.n, R).spb * c.n * R * sizeof(cplx<float>) > 200 * 1024)
+    throw Error(DDTM_ERR_ARG, "coarse_even: " + std::to_string(R) + " right-hand sides of " + std::to_string(c.n) +
+                                  " dofs exceed the shared-memory stage");
+  coarse_split(c, t, nullptr, v, c.nbr_eo.as<int>(), c.even.as<int>(), (int)c.h_even.size(), R, 0.f, v ? 2 : 0, sh, 0.f,
+               c.Dinv.as<float2>(), rhs, sr, st);
 }
 
 void launch_parity_copy(const CoarseLevel& c, int parity, cplx<float>* compact, cplx<float>* full, int R, int dir,

@@ -1,5 +1,5 @@
-// Launch shape of the SIMT coarse stencil kernels (k_coarse_apply,
-// k_coarse_even in coarse.cu).  Plain host C++, no CUDA types, so that a host
+// Launch shape of the SIMT coarse stencil kernel of single hops
+// (k_coarse_hop in coarse.cu).  Plain host C++, no CUDA types, so that a host
 // unit test can compile it alone and check every (n, R) it may meet.
 //
 // A site of the coarse lattice (n = 2 nv rows) with R right-hand sides is
