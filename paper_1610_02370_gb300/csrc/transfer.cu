@@ -700,11 +700,14 @@ __device__ __forceinline__ void cmma(float (&cr)[4], float (&ci)[4], const AFrag
 }
 
 // c = P^dagger psi.  One CTA per (aggregate, s) and 8 NT right-hand sides; its warps share the depth (runs of 4 sites
-// of a component), every warp forms all rows, and the partial sums meet in shared memory.
+// of a component), every warp forms all rows, and the partial sums meet in shared memory.  Bound by the latency of the P
+// loads: two CTAs per SM with 80 registers and a few spilled values take 464 us for 12 right-hand sides of 24^3 x 48 and
+// 24 vectors, one with 100 registers 524; beyond 32 vectors the accumulators need all registers of one.
 static const int RM_WARPS = 12;
 template <int MT, int NT>
-__global__ void __launch_bounds__(32 * RM_WARPS) k_restrict_mma(cplx<float>* __restrict__ c, Spinor<PREC_F16> psi, size_t fstride, long V,
-                                                               const __half2* __restrict__ P, int nv, int R, int Rs) {
+__global__ void __launch_bounds__(32 * RM_WARPS, MT <= 2 ? 2 : 1)
+    k_restrict_mma(cplx<float>* __restrict__ c, Spinor<PREC_F16> psi, size_t fstride, long V, const __half2* __restrict__ P,
+                   int nv, int R, int Rs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* part = reinterpret_cast<float2*>(smem_raw);  // [warp][16 MT][8 NT + 1]
   const int Vb = psi.Vb, blk = blockIdx.x >> 1, s = blockIdx.x & 1, r0 = blockIdx.y * 8 * NT;
