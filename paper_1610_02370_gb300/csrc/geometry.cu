@@ -400,8 +400,7 @@ __global__ void k_spinor_from_canon(Spinor<P> out, const double2* __restrict__ i
 // memory, so that the 192 contiguous bytes of a canonical site are written by 12 neighbouring threads, in full
 // sectors.  Bound by HBM: 39 us per FP32 field of 24^3 x 48 (191 MB, 4.9 TB/s); one thread per site, writing its
 // 192 bytes piecewise, took 77.
-static const int LT = 256;
-template <int P>
+template <int P, int LT>
 __global__ void __launch_bounds__(LT) k_spinor_to_canon(Spinor<P> in, double2* __restrict__ out, CanonMap m, long V) {
   typedef typename Prec<P>::real R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -453,18 +452,25 @@ static void spinor_from_canon_t(const FineGeom& g, void* d, float* nrm, const do
     CKL("spinor_from_canon");
   }
 }
-template <int P>
+template <int P, int LT>
 static void spinor_to_canon_t(const FineGeom& g, const void* d, const float* nrm, double* out, int R, cudaStream_t s) {
   const size_t smem = 12 * (LT + 1) * sizeof(cplx<typename Prec<P>::real>);
-  set_dynamic_smem((const void*)k_spinor_to_canon<P>, smem);
+  set_dynamic_smem((const void*)k_spinor_to_canon<P, LT>, smem);
   typedef typename Prec<P>::store2 S;
   for (int r = 0; r < R; r += 65535) {  // grid.y
     const size_t o = (size_t)r * 12 * g.V;
-    k_spinor_to_canon<P><<<dim3(grid_for(g.V, LT), R - r < 65535 ? R - r : 65535), LT, smem, s>>>(
+    k_spinor_to_canon<P, LT><<<dim3(grid_for(g.V, LT), R - r < 65535 ? R - r : 65535), LT, smem, s>>>(
         Spinor<P>{(S*)d + o, nrm ? (float*)nrm + (size_t)r * g.V : nullptr, g.Vb}, reinterpret_cast<double2*>(out) + o,
         make_map(g), g.V);
     CKL("spinor_to_canon");
   }
+}
+// Tiles of 256 sites, or of 32 while those make fewer than two CTAs per SM: the stores and the FP64 conversions of a
+// tile then are what a small field waits for (FP64 field of 8192 sites: 17.6 us with 256, 6.3 with 32).
+template <int P>
+static void spinor_to_canon_p(const FineGeom& g, const void* d, const float* nrm, double* out, int R, cudaStream_t s) {
+  if ((long)grid_for(g.V, 256) * R < 304) spinor_to_canon_t<P, 32>(g, d, nrm, out, R, s);
+  else spinor_to_canon_t<P, 256>(g, d, nrm, out, R, s);
 }
 
 void launch_spinor_from_canon(const FineGeom& g, int prec, void* d, float* nrm, const double* in, cudaStream_t s, int R) {
@@ -476,9 +482,9 @@ void launch_spinor_from_canon(const FineGeom& g, int prec, void* d, float* nrm, 
 
 void launch_spinor_to_canon(const FineGeom& g, int prec, const void* d, const float* nrm, double* out, cudaStream_t s, int R) {
   ScopedTimer timer_("layout_out", s, R);
-  if (prec == PREC_F64) spinor_to_canon_t<PREC_F64>(g, d, nrm, out, R, s);
-  else if (prec == PREC_F32) spinor_to_canon_t<PREC_F32>(g, d, nrm, out, R, s);
-  else spinor_to_canon_t<PREC_F16>(g, d, nrm, out, R, s);
+  if (prec == PREC_F64) spinor_to_canon_p<PREC_F64>(g, d, nrm, out, R, s);
+  else if (prec == PREC_F32) spinor_to_canon_p<PREC_F32>(g, d, nrm, out, R, s);
+  else spinor_to_canon_p<PREC_F16>(g, d, nrm, out, R, s);
 }
 
 void launch_links_from_canon(const FineGeom& g, double* out, const double* U, cudaStream_t s) {
