@@ -519,8 +519,11 @@ __global__ void __launch_bounds__(VB, 3)
 // quarter of each sector) and their latency at 16 warps per SM.  Not taken: 128 threads per block with the two
 // parities in turn (703 / 790, one 118 / 83), the faces staged in shared memory first (1020 / 822), three pairs per CTA
 // sharing the operator through L1 (874 / 834).
-template <int P, typename V>
-__global__ void __launch_bounds__(256, vlanes<V>() == 2 ? 2 : 3)
+// One right-hand side: three CTAs per SM (80 registers), or two without spills and with more loads in flight while all
+// CTAs of the launch are resident with two (three FP32 applications and an export at 8192 sites 39 us with three, 35
+// with two).
+template <int P, typename V, int MINB>
+__global__ void __launch_bounds__(256, MINB)
     k_dslash_b4(Spinor<P> yf, Spinor<P> xf, const typename Prec<P>::store2* __restrict__ U,
                 const typename Prec<P>::store2* __restrict__ C, Geo g, float mu, int nrhs, size_t fstride, long Vs,
                 int chunk) {
@@ -567,13 +570,13 @@ static Geo make_geo(const FineGeom& g) {
 static bool dslash_blk_ok(const FineGeom& g, int prec) { return prec != PREC_F64 && g.Vb == 256; }
 
 static const int B4_CHUNK = 64;
-template <int P, typename V>
+template <int P, typename V, int MINB>
 static void dslash_b4_t(const FineGeom& g, Spinor<P> Y, Spinor<P> X, const typename Prec<P>::store2* U,
                         const typename Prec<P>::store2* C, double mu, int nrhs, cudaStream_t s) {
   const size_t smem = 2 * 12 * B4_VH * sizeof(cv<V>);
-  set_dynamic_smem((const void*)k_dslash_b4<P, V>, smem);
+  set_dynamic_smem((const void*)k_dslash_b4<P, V, MINB>, smem);
   const unsigned groups = (nrhs + vlanes<V>() - 1) / vlanes<V>();
-  k_dslash_b4<P, V><<<(unsigned)g.Nb * groups, 256, smem, s>>>(Y, X, U, C, make_geo(g), (float)mu, nrhs,
+  k_dslash_b4<P, V, MINB><<<(unsigned)g.Nb * groups, 256, smem, s>>>(Y, X, U, C, make_geo(g), (float)mu, nrhs,
                                                               (size_t)g.V * 12, g.V, B4_CHUNK);
   CKL("dslash_b4");
 }
@@ -584,8 +587,8 @@ static void dslash_blk_t(const FineGeom& g, void* y, float* ynrm, const void* x,
   typedef typename Prec<P>::store2 S;
   Spinor<P> Y{(S*)y, ynrm, g.Vb}, X{(S*)x, (float*)xnrm, g.Vb};
   if (g.b[0] == 4 && g.b[1] == 4 && g.b[2] == 4 && g.b[3] == 4) {
-    if (nrhs > 1) dslash_b4_t<P, float2>(g, Y, X, (const S*)links, (const S*)clover, mu, nrhs, s);
-    else dslash_b4_t<P, float>(g, Y, X, (const S*)links, (const S*)clover, mu, nrhs, s);
+    auto go = nrhs > 1 ? dslash_b4_t<P, float2, 2> : g.Nb <= 304 ? dslash_b4_t<P, float, 2> : dslash_b4_t<P, float, 3>;
+    go(g, Y, X, (const S*)links, (const S*)clover, mu, nrhs, s);
     return;
   }
   k_dslash_blk<P, 256><<<g.Nb, 256, 0, s>>>(Y, X, Links<P>{(const S*)links, g.Vb}, Clover<P>{(const S*)clover, g.Vb},
