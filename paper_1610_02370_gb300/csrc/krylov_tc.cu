@@ -9,7 +9,8 @@
 //   B  w -= sum_i h_i V_i (w in registers), norms   -> barrier
 //   C  V_next = w / ||w|| in FP16; one warp per right-hand side does the Givens update
 // The grid is one wave, one CTA per SM at most (cooperative launch); barrier waits are bounded and a timeout sets
-// *err like the tensor-core passes.
+// *err like the tensor-core passes.  Every barrier has a counter of its own, clear when its first CTA arrives: a step
+// clears the counters that its later barriers make free, and the launch of a cycle's first step (no basis vectors) clears all.
 // Bound by reading the basis twice (HBM, or L2 where it fits) and, where it is small, by the latency of three
 // barriers and of the FP64 tail (hence inv_sqrt and the warps that share a tile).  Measured per iteration over a
 // solve, between events: 24^3 x 48, 12 right-hand sides, 59 vectors on average: 69 us; before (multi-dot,
@@ -500,6 +501,9 @@ void launch_gs_step(const ImgVec& v, const void* V, size_t ldv, int nvec, float*
   g.err = b.err;
   g.xb_off = (int)gs_xb_off(v, nvec, p);
   g.turn_off = (int)gs_turn_off(v, nvec, p);
+  // The last step of a cycle leaves the counter of its norm barrier at the number of CTAs; steps with basis vectors clear it
+  // themselves behind their first barrier, a step without any has no barrier before that one.  (Also after a timeout.)
+  if (nvec == 0) CK(cudaMemsetAsync(b.bar, 0, 3 * sizeof(unsigned), st));
   void* args[] = {(void*)&g};
   CK(cudaLaunchCooperativeKernel(gs_kernel(p.nt), dim3(p.ctas), dim3(p.nt), args, gs_smem(v, nvec, p), st));
   CKL("gs_step");

@@ -17,7 +17,7 @@ struct ImgVec {
 };
 
 // Work buffers of the Arnoldi step: partial sums over the launch's CTAs, the coefficients h[i * R + r], grid
-// barrier counters (cleared by the caller before the first step of a solve) and the timeout flag.
+// barrier counters (cleared by the launch of a step without basis vectors) and the timeout flag.
 struct GsBuffers {
   float2* part;
   double2* h;

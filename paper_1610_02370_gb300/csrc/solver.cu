@@ -459,7 +459,6 @@ static int gmres_img(ddtm_ctx* c, CoarseLevel& L, const ImgVec& v, int ctas, con
   c->events("cgi", ev);
   CK(cudaMemsetAsync(x, 0, ne * sizeof(float), c->stream));
   CK(cudaMemsetAsync(w, 0, ne * sizeof(float), c->stream));  // its padding entries stay zero
-  CK(cudaMemsetAsync(gb.bar, 0, 3 * sizeof(unsigned), c->stream));
   std::vector<double> est(R, 0.0);
   // the estimates of slot, once their kernel has run; true when every system has converged
   auto converged = [&](int slot) {
