@@ -564,8 +564,10 @@ int coarse_eo_solve(ddtm_ctx* c, cplx<float>* x_full, const cplx<float>* b_full,
   launch_parity_copy(L, 1, bo, (cplx<float>*)b_full, Rc, 0, c->stream);
   launch_coarse_even(L, te, be, nullptr, Rc, 1.f, 0.f, c->stream);                 // te = D_ee^-1 eta_e
   launch_coarse_apply_odd(L, bo, nullptr, te, Rc, mu_c, 2, -1.f, 1.f, c->stream);   // rhat = eta_o - D_oe te
-  char ok[96];  // what the operator's launch arguments depend on besides buffers
-  snprintf(ok, sizeof(ok), "eo|mu%.17g|p%d|lev%p", mu_c, L.prec, (const void*)&L);
+  // what the operator's launch arguments depend on besides buffers: the dofs too, since a hierarchy of fewer test vectors
+  // reuses the buffers of the one before, and its vectors may have as many padded entries
+  char ok[112];
+  snprintf(ok, sizeof(ok), "eo|mu%.17g|n%d|p%d|lev%p", mu_c, L.n, L.prec, (const void*)&L);
   const ImgVec v{tc_geom(L.n, Rc), (int)no};
   const int ctas = L.prec == PREC_F16 && tol >= 1e-3 ? gs_ctas(v, restart) : 0;
   if (ctas > 0) {

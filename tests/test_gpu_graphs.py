@@ -88,3 +88,49 @@ def test_autotuner_choice_leaves_results_unchanged(lib):
     finally:
         lib.ddtm_set_option(ctx, "autotune", 1)
         lib.ddtm_destroy(ctx)
+
+
+@pytest.mark.parametrize("coarse_prec", [1, 2])
+def test_graphs_follow_the_number_of_test_vectors(lib, coarse_prec):
+    """A context that goes from 24 to 20 and back to 24 test vectors keeps its buffers (they fit), so nothing but the key of a
+    cached graph tells the hierarchies apart (48 and 40 dofs, both padded to 48): every solve has the bits of a
+    fresh context and of direct launches."""
+    dims, mu = (8, 8, 8, 16), 0.02
+    U = synth.gauge_field(dims, 0.2, seed=71).cuda()
+    v = synth.gaussian_vectors((24, 8, 16, 8, 8, 4, 3), seed=72).cuda()
+
+    def context():
+        ctx = lib.ddtm_create(dims, (4, 4, 4, 4), 0)
+        lib.ddtm_load_gauge(ctx, U, 0.134, 1.5755)
+        return ctx
+
+    def solve(ctx, nv, graphs):
+        p = lib.ddtm_get_params(ctx)
+        p.nv[0], p.coarse_prec, p.coarse_tol = nv, coarse_prec, 1e-2
+        lib.ddtm_set_params(ctx, p)
+        lib.ddtm_set_test_vectors(ctx, 0, v[:nv].contiguous(), nv)
+        lib.ddtm_set_option(ctx, "graphs", graphs)
+        b = synth.gaussian_vectors((12, 2, 4, 2, 2, 2 * nv), seed=73).cuda()
+        out = []
+        for _ in range(3):  # direct, captured, replayed
+            x = torch.zeros_like(b)
+            iters, code = lib.ddtm_coarse_solve_batch(ctx, x, b, 12, mu)
+            assert code == lib.OK and iters > 0
+            out.append(x)
+        assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+        return out[0]
+
+    want = {}
+    for nv in (24, 20):
+        fresh = context()
+        try:
+            want[nv] = solve(fresh, nv, 0)
+        finally:
+            lib.ddtm_destroy(fresh)
+    ctx = context()  # no allocation by any other context from here on: those would drop the graphs
+    try:
+        for nv in (24, 20, 24):
+            assert torch.equal(solve(ctx, nv, 1), want[nv]), nv
+        assert lib.ddtm_get_option(ctx, "graphs_cached") > 0
+    finally:
+        lib.ddtm_destroy(ctx)
