@@ -741,24 +741,23 @@ __global__ void k_parity_copy(cplx<float>* __restrict__ compact, cplx<float>* __
   else full[f] = compact[t];
 }
 
-// canonical FP64 coarse vector c[site * n + k] <-> column r of an interleaved
-// FP32 batch v[(site * n + k) * R + r] (dir 0: c -> v, dir 1: v -> c)
-// Canonical FP64 coarse vectors c[r][nc] <-> columns r0 ... r0 + nr - 1 of the interleaved batch v[nc][R]: tiles of
-// IL_T entries x IL_R columns turned through shared memory, so that both sides are contiguous.
+// Canonical FP64 coarse vectors c[r][nc] <-> columns r0 ... r0 + nr - 1 of the interleaved FP32 batch v[nc][R] (dir 0: c ->
+// v, dir 1: v -> c): tiles of IL_T entries x IL_R columns turned through shared memory, so that both sides are contiguous.
 static const int IL_T = 64, IL_R = 32;
-__global__ void __launch_bounds__(256) k_coarse_interleave(float2* __restrict__ v, double2* __restrict__ c, size_t nc, int r0,
+template <bool A16>
+__global__ void __launch_bounds__(256) k_coarse_interleave(float2* __restrict__ v, double* __restrict__ c, size_t nc, int r0,
                                                            int nr, int R, int dir) {
   __shared__ float2 t[IL_T * (IL_R + 1)];
   const size_t e0 = (size_t)blockIdx.x * IL_T;
   const int q0 = blockIdx.y * IL_R, nq = nr - q0 < IL_R ? nr - q0 : IL_R;
   const int ne = nc - e0 < (size_t)IL_T ? (int)(nc - e0) : IL_T;
-  c += (size_t)q0 * nc + e0;
+  c += 2 * ((size_t)q0 * nc + e0);
   v += e0 * R + r0 + q0;
   if (dir == 0) {
     for (int k = threadIdx.x; k < IL_T * nq; k += blockDim.x) {
       const int q = k / IL_T, e = k - q * IL_T;
       if (e < ne) {
-        const double2 a = c[(size_t)q * nc + e];
+        const double2 a = ld_canon<A16>(c, (size_t)q * nc + e);
         t[e * (IL_R + 1) + q] = make_float2((float)a.x, (float)a.y);
       }
     }
@@ -777,7 +776,7 @@ __global__ void __launch_bounds__(256) k_coarse_interleave(float2* __restrict__ 
       const int q = k / IL_T, e = k - q * IL_T;
       if (e < ne) {
         const float2 z = t[e * (IL_R + 1) + q];
-        c[(size_t)q * nc + e] = make_double2((double)z.x, (double)z.y);
+        st_canon<A16>(c, (size_t)q * nc + e, (double)z.x, (double)z.y);
       }
     }
   }
@@ -916,8 +915,9 @@ void launch_coarse_interleave(const CoarseLevel& c, cplx<float>* v, double* cano
   const size_t nc = (size_t)c.Nc * c.n;
   for (int q = 0; q < nr; q += 65535 * IL_R) {  // grid.y
     const int n = nr - q < 65535 * IL_R ? nr - q : 65535 * IL_R;
-    k_coarse_interleave<<<dim3((unsigned)((nc + IL_T - 1) / IL_T), (n + IL_R - 1) / IL_R), 256, 0, st>>>(
-        reinterpret_cast<float2*>(v), reinterpret_cast<double2*>(canon) + (size_t)q * nc, nc, r + q, n, R, dir);
+    auto kernel = canon_a16(canon) ? k_coarse_interleave<true> : k_coarse_interleave<false>;
+    kernel<<<dim3((unsigned)((nc + IL_T - 1) / IL_T), (n + IL_R - 1) / IL_R), 256, 0, st>>>(
+        reinterpret_cast<float2*>(v), canon + 2 * (size_t)q * nc, nc, r + q, n, R, dir);
     CKL("coarse_interleave");
   }
 }

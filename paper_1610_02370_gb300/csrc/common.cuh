@@ -72,6 +72,22 @@ __device__ __forceinline__ cplx<float> ld(const __half2* p) {
   float2 f = __half22float2(v);
   return cplx<float>(f.x, f.y);
 }
+// complex entry i of a canonical coarse vector of the caller, whose array is aligned to 8 bytes at least: one 16-byte access
+// (A16) where the array allows it, two of 8 bytes otherwise
+template <bool A16> __device__ __forceinline__ double2 ld_canon(const double* p, size_t i) {
+  if (A16) return reinterpret_cast<const double2*>(p)[i];
+  return make_double2(p[2 * i], p[2 * i + 1]);
+}
+template <bool A16> __device__ __forceinline__ void st_canon(double* p, size_t i, double re, double im) {
+  if (A16) {
+    reinterpret_cast<double2*>(p)[i] = make_double2(re, im);
+  } else {
+    p[2 * i] = re;
+    p[2 * i + 1] = im;
+  }
+}
+inline bool canon_a16(const double* p) { return ((uintptr_t)p & 15) == 0; }
+
 // plain (non-__ldg) loads for buffers written earlier in the same kernel
 __device__ __forceinline__ cplx<double> ldw(const double2* p) { double2 v = *p; return cplx<double>(v.x, v.y); }
 __device__ __forceinline__ cplx<float> ldw(const float2* p) { float2 v = *p; return cplx<float>(v.x, v.y); }

@@ -568,12 +568,13 @@ __device__ __forceinline__ size_t img_entry(int r, int q, int n, int b_half, int
   const int s = q / n, k = q - s * n;
   return (size_t)s * b_half + (size_t)(r >> 2) * g_half + (k >> 3) * 64 + (r & 3) * 16 + (k & 7);
 }
-__global__ void k_img_from_canon(__half* __restrict__ image, float* __restrict__ img, const double2* __restrict__ x, int nc,
-                                 int n, int b_half, int g_half, int R) {
+template <bool A16>
+__global__ void k_img_from_canon(__half* __restrict__ image, float* __restrict__ img, const double* __restrict__ x, int nc, int n,
+                                 int b_half, int g_half, int R) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nc) return;
   for (int r = blockIdx.y; r < R; r += gridDim.y) {
-    const double2 z = __ldg(x + (size_t)r * nc + q);
+    const double2 z = ld_canon<A16>(x, (size_t)r * nc + q);
     const float re = (float)z.x, im = (float)z.y;
     const size_t o = img_entry(r, q, n, b_half, g_half);
     img[o] = re;
@@ -582,12 +583,13 @@ __global__ void k_img_from_canon(__half* __restrict__ image, float* __restrict__
     image[o + 8] = __float2half_rn(im);
   }
 }
-__global__ void k_img_to_canon(double2* __restrict__ y, const float* __restrict__ img, int nc, int n, int b_half, int g_half, int R) {
+template <bool A16>
+__global__ void k_img_to_canon(double* __restrict__ y, const float* __restrict__ img, int nc, int n, int b_half, int g_half, int R) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nc) return;
   for (int r = blockIdx.y; r < R; r += gridDim.y) {
     const size_t o = img_entry(r, q, n, b_half, g_half);
-    y[(size_t)r * nc + q] = make_double2((double)img[o], (double)img[o + 8]);
+    st_canon<A16>(y, (size_t)r * nc + q, (double)img[o], (double)img[o + 8]);
   }
 }
 
@@ -633,15 +635,17 @@ void launch_img_from_canon(const ImgVec& v, void* image, float* img, const doubl
     CK(cudaMemsetAsync(image, 0, v.entries() * sizeof(__half), st));
     CK(cudaMemsetAsync(img, 0, v.entries() * sizeof(float), st));
   }
-  k_img_from_canon<<<dim3((nc + 255) / 256, v.t.R < 65535 ? v.t.R : 65535), 256, 0, st>>>(
-      (__half*)image, img, (const double2*)x, nc, v.t.n, v.t.b_bytes / 2, v.t.sbo / 2, v.t.R);
+  auto kernel = canon_a16(x) ? k_img_from_canon<true> : k_img_from_canon<false>;
+  kernel<<<dim3((nc + 255) / 256, v.t.R < 65535 ? v.t.R : 65535), 256, 0, st>>>((__half*)image, img, x, nc, v.t.n,
+                                                                              v.t.b_bytes / 2, v.t.sbo / 2, v.t.R);
   CKL("img_from_canon");
 }
 void launch_img_to_canon(const ImgVec& v, double* y, const float* img, cudaStream_t st) {
   ScopedTimer timer_("img_order", st, v.t.R);
   const int nc = v.nsites * v.t.n;
-  k_img_to_canon<<<dim3((nc + 255) / 256, v.t.R < 65535 ? v.t.R : 65535), 256, 0, st>>>((double2*)y, img, nc, v.t.n,
-                                                                                       v.t.b_bytes / 2, v.t.sbo / 2, v.t.R);
+  auto kernel = canon_a16(y) ? k_img_to_canon<true> : k_img_to_canon<false>;
+  kernel<<<dim3((nc + 255) / 256, v.t.R < 65535 ? v.t.R : 65535), 256, 0, st>>>(y, img, nc, v.t.n, v.t.b_bytes / 2,
+                                                                              v.t.sbo / 2, v.t.R);
   CKL("img_to_canon");
 }
 void launch_img_half(const ImgVec& v, void* out, const float* in, cudaStream_t st) {
