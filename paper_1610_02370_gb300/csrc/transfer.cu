@@ -576,6 +576,9 @@ static const int PP_NP = 3;  // pairs per CTA of k_prolong_pair
 // vectors, FP32: 3, 3, 256, 2: 532 us; 3, 3, 256, 3: 667; 3, 2, 384, 2: 550; 6, 2, 384, 1: 616; 6, 1, 768, 1: 718
 // (scalar arithmetic, two P entries in flight and the chunks of a block far apart: 1025).  The prolongation, 3 pairs:
 // 561 us (815).  Both are bound by the latency of the P loads and shared memory; P and the fields alone take 340 us.
+// FP16 fields with the FP16 copy of P (the solver's): 552 and 528 us.  TF32 matrix instructions with the FP32 operand as
+// hi + lo took 469 and 608 us (one right-hand side 248 and 309, here 757 and 264), but the unit cuts its sums off towards
+// zero: 1.2e-6 against 64 bits where these kernels have 1.9e-7, and with the cut parts fetched back they took 929 and 986.
 static const int RP_NP = 3, RP_OW = 3, RP_NT = 256, RP_MINB = 2;
 template <int PI, typename PS>
 static void restrict_p(const FineGeom& g, cplx<float>* c, Spinor<PI> f, size_t fstride, const PS* P, int nv, int R,
@@ -641,232 +644,11 @@ static void prolong_t(const FineGeom& g, int pout, void* x, float* xn, const cpl
   CKL("prolong");
 }
 
-// ---- restriction and prolongation of FP16 fields with the FP16 copy of P (the smoother's precision) -----------
-// Both are dense contractions per aggregate and chirality half s, with R right-hand sides as columns:
-//   c[i][r] = sum over (component, site) conj(P_i) psi_r        (nv x R, depth 6 Vb)
-//   x_r(component, site) = sum_i P_i e[i][r]                    (6 Vb x R, depth nv)
-// done by mma.sync m16n8k8 in TF32: P's FP16 entries are exact in TF32, the other operand goes in as hi + lo (21 bits),
-// sums are FP32.  The unit's sums carry about 2e-6 (measured with FP32 operands in three products, against 3e-7 of
-// the FP32 kernels above, which therefore keep FP32 fields); beside the 5e-4 of the FP16 operands that is nothing.
-// Fragments are loaded straight from memory: P once per 16 right-hand sides, psi once.  A complex product takes 4 of
-// the 8 depths for the real and 4 for the imaginary parts.  Every right-hand side is a column of its own, so a batch
-// gives the same bits as its right-hand sides one by one.
-// 16^3 x 32, 12 right-hand sides, 24 vectors: restriction 135 us, prolongation 161 us (SIMT kernels above 292, 202).
-__device__ __forceinline__ uint32_t tf32_of(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ uint32_t neg_u(uint32_t x) { return x ^ 0x80000000u; }
-__device__ __forceinline__ void mma_t(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-// a fragment of A: FP16 complex entries of rows g and g + 8, one k each
-struct AFrag {
-  uint32_t gr, gi, hr, hi;
-};
-__device__ __forceinline__ AFrag a_frag(cplx<float> g, cplx<float> h) {
-  return AFrag{__float_as_uint(g.re), __float_as_uint(g.im), __float_as_uint(h.re), __float_as_uint(h.im)};
-}
-// a fragment of B: one complex entry as hi + lo
-struct BFrag {
-  uint32_t re, im, rel, iml;
-};
-__device__ __forceinline__ BFrag b_frag(cplx<float> z) {
-  BFrag f;
-  f.re = tf32_of(z.re);
-  f.im = tf32_of(z.im);
-  f.rel = tf32_of(z.re - __uint_as_float(f.re));
-  f.iml = tf32_of(z.im - __uint_as_float(f.im));
-  return f;
-}
-// (cr, ci) += conj(A) B (CONJ) or A B
-template <bool CONJ>
-__device__ __forceinline__ void cmma(float (&cr)[4], float (&ci)[4], const AFrag& a, const BFrag& b) {
-  const uint32_t ngi = neg_u(a.gi), nhi = neg_u(a.hi);
-  if (CONJ) {  // re: ar br + ai bi; im: -ai br + ar bi
-    mma_t(cr, a.gr, a.hr, a.gi, a.hi, b.re, b.im);
-    mma_t(ci, ngi, nhi, a.gr, a.hr, b.re, b.im);
-    mma_t(cr, a.gr, a.hr, a.gi, a.hi, b.rel, b.iml);
-    mma_t(ci, ngi, nhi, a.gr, a.hr, b.rel, b.iml);
-  } else {  // re: ar br - ai bi; im: ai br + ar bi
-    mma_t(cr, a.gr, a.hr, ngi, nhi, b.re, b.im);
-    mma_t(ci, a.gi, a.hi, a.gr, a.hr, b.re, b.im);
-    mma_t(cr, a.gr, a.hr, ngi, nhi, b.rel, b.iml);
-    mma_t(ci, a.gi, a.hi, a.gr, a.hr, b.rel, b.iml);
-  }
-}
-
-// c = P^dagger psi.  One CTA per (aggregate, s) and 8 NT right-hand sides; its warps share the depth (runs of 4 sites
-// of a component), every warp forms all rows, and the partial sums meet in shared memory.  Bound by the latency of the P
-// loads: two CTAs per SM with 80 registers and a few spilled values take 464 us for 12 right-hand sides of 24^3 x 48 and
-// 24 vectors, one with 100 registers 524; beyond 32 vectors the accumulators need all registers of one.
-static const int RM_WARPS = 12;
-template <int MT, int NT>
-__global__ void __launch_bounds__(32 * RM_WARPS, MT <= 2 ? 2 : 1)
-    k_restrict_mma(cplx<float>* __restrict__ c, Spinor<PREC_F16> psi, size_t fstride, long V, const __half2* __restrict__ P,
-                   int nv, int R, int Rs) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* part = reinterpret_cast<float2*>(smem_raw);  // [warp][16 MT][8 NT + 1]
-  const int Vb = psi.Vb, blk = blockIdx.x >> 1, s = blockIdx.x & 1, r0 = blockIdx.y * 8 * NT;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  float cr[MT][NT][4], ci[MT][NT][4];
-#pragma unroll
-  for (int m = 0; m < MT; m++)
-#pragma unroll
-    for (int q = 0; q < NT; q++)
-#pragma unroll
-      for (int k = 0; k < 4; k++) cr[m][q][k] = ci[m][q][k] = 0.f;
-  const __half2* pg[MT];
-  const __half2* ph[MT];
-#pragma unroll
-  for (int m = 0; m < MT; m++) {  // rows beyond nv repeat the last one and are not stored
-    const int i0 = 16 * m + g < nv ? 16 * m + g : nv - 1, i1 = 16 * m + g + 8 < nv ? 16 * m + g + 8 : nv - 1;
-    pg[m] = P + ((size_t)(blk * 2 + s) * nv + i0) * 6 * Vb + t;
-    ph[m] = P + ((size_t)(blk * 2 + s) * nv + i1) * 6 * Vb + t;
-  }
-  const __half2* f[NT];
-  const float* fn[NT];
-#pragma unroll
-  for (int q = 0; q < NT; q++) {  // columns beyond R repeat the last one
-    const int r = r0 + 8 * q + g < R ? r0 + 8 * q + g : R - 1;
-    f[q] = psi.d + (size_t)r * fstride + ((size_t)blk * 12 + 6 * s) * Vb + t;
-    fn[q] = psi.nrm + (size_t)r * V + (size_t)blk * Vb + t;
-  }
-  const int ks = 6 * Vb / 4, kb = warp * ks / RM_WARPS, ke = (warp + 1) * ks / RM_WARPS;
-  int site = 4 * kb % Vb;
-#pragma unroll 4
-  for (int k = kb; k < ke; k++) {
-    const int e = 4 * k;  // component * Vb + site of the run
-    BFrag b[NT];
-#pragma unroll
-    for (int q = 0; q < NT; q++) {
-      b[q] = b_frag(__ldg(fn[q] + site) * ld(f[q] + e));
-    }
-#pragma unroll
-    for (int m = 0; m < MT; m++) {
-      const AFrag a = a_frag(ld(pg[m] + e), ld(ph[m] + e));
-#pragma unroll
-      for (int q = 0; q < NT; q++) cmma<true>(cr[m][q], ci[m][q], a, b[q]);
-    }
-    site = site + 4 < Vb ? site + 4 : 0;
-  }
-  constexpr int LD = 8 * NT + 1;
-#pragma unroll
-  for (int m = 0; m < MT; m++)
-#pragma unroll
-    for (int q = 0; q < NT; q++)
-#pragma unroll
-      for (int k = 0; k < 4; k++)
-        part[((size_t)warp * 16 * MT + 16 * m + g + 8 * (k >> 1)) * LD + 8 * q + 2 * t + (k & 1)] = make_float2(cr[m][q][k], ci[m][q][k]);
-  __syncthreads();
-  for (int o = threadIdx.x; o < 16 * MT * 8 * NT; o += blockDim.x) {
-    const int i = o / (8 * NT), r = o - i * 8 * NT;
-    if (i >= nv || r0 + r >= R) continue;
-    float re = 0.f, im = 0.f;
-#pragma unroll
-    for (int w = 0; w < RM_WARPS; w++) {
-      const float2 p = part[((size_t)w * 16 * MT + i) * LD + r];
-      re += p.x;
-      im += p.y;
-    }
-    c[((size_t)blk * 2 * nv + s * nv + i) * Rs + r0 + r] = cplx<float>(re, im);
-  }
-}
-
-// x_r = P e_r (add = 0) or x_r += P e_r.  One CTA per aggregate and 8 right-hand sides (neighbouring CTAs share the
-// aggregate's P through L2); a warp takes 16 sites at a time and all 12 components of them (FP16 storage keeps
-// one scale per site), e_B comes from shared memory.
-__global__ void __launch_bounds__(128, 3) k_prolong_mma(Spinor<PREC_F16> x, size_t fstride, long V, const cplx<float>* __restrict__ e,
-                                                        const __half2* __restrict__ P, int nv, int R, int Rs, int add) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* se = reinterpret_cast<float2*>(smem_raw);  // [2][nv4][9], rows beyond nv are zero
-  const int Vb = x.Vb, nchunk = (R + 7) / 8, blk = blockIdx.x / nchunk, r0 = (blockIdx.x - blk * nchunk) * 8;
-  const int nv4 = (nv + 3) / 4 * 4, n = 2 * nv;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, nw = blockDim.x >> 5;
-  for (int k = threadIdx.x; k < 2 * nv4 * 8; k += blockDim.x) {
-    const int r = k & 7, o = k >> 3, s = o / nv4, i = o - s * nv4;
-    const cplx<float> z = i < nv && r0 + r < R ? e[((size_t)blk * n + s * nv + i) * Rs + r0 + r] : cplx<float>(0, 0);
-    se[o * 9 + r] = make_float2(z.re, z.im);
-  }
-  __syncthreads();
-  for (int x0 = 16 * warp; x0 < Vb; x0 += 16 * nw) {
-    float cr[12][4], ci[12][4];
-#pragma unroll
-    for (int c = 0; c < 12; c++)
-#pragma unroll
-      for (int k = 0; k < 4; k++) cr[c][k] = ci[c][k] = 0.f;
-#pragma unroll
-    for (int s = 0; s < 2; s++)
-#pragma unroll 1
-      for (int i0 = 0; i0 < nv; i0 += 4) {
-        const float2 ev = se[(s * nv4 + i0 + t) * 9 + g];
-        const BFrag b = b_frag(cplx<float>(ev.x, ev.y));
-        const int i = i0 + t < nv ? i0 + t : nv - 1;  // beyond nv e is zero
-        const __half2* p = P + ((size_t)(blk * 2 + s) * nv + i) * 6 * Vb + x0 + g;
-        cplx<float> pa[6], pb[6];
-#pragma unroll
-        for (int c = 0; c < 6; c++) {
-          pa[c] = ld(p + (size_t)c * Vb);
-          pb[c] = ld(p + (size_t)c * Vb + 8);
-        }
-#pragma unroll
-        for (int c = 0; c < 6; c++) cmma<false>(cr[6 * s + c], ci[6 * s + c], a_frag(pa[c], pb[c]), b);
-      }
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const int r = r0 + 2 * t + (k & 1), loc = x0 + g + 8 * (k >> 1);
-      if (r >= R) continue;
-      Spinor<PREC_F16> f = x;
-      f.d += (size_t)r * fstride;
-      f.nrm += (size_t)r * V;
-      cplx<float> out[12];
-      if (add) f.loadw(blk, loc, out);
-#pragma unroll
-      for (int c = 0; c < 12; c++) {
-        const cplx<float> a(cr[c][k], ci[c][k]);
-        out[c] = add ? out[c] + a : a;
-      }
-      f.store(blk, loc, out);
-    }
-  }
-}
-
-template <int MT>
-static void restrict_mma_m(const FineGeom& g, cplx<float>* c, Spinor<PREC_F16> f, const __half2* P, int nv, int R, int Rs, cudaStream_t st) {
-  const int NT = R <= 8 ? 1 : 2;
-  const size_t smem = (size_t)RM_WARPS * 16 * MT * (8 * NT + 1) * sizeof(float2);
-  const void* k = NT == 1 ? (const void*)k_restrict_mma<MT, 1> : (const void*)k_restrict_mma<MT, 2>;
-  set_dynamic_smem(k, smem);
-  const dim3 grid(g.Nb * 2, (R + 8 * NT - 1) / (8 * NT));
-  if (NT == 1) k_restrict_mma<MT, 1><<<grid, 32 * RM_WARPS, smem, st>>>(c, f, (size_t)g.V * 12, g.V, P, nv, R, Rs);
-  else k_restrict_mma<MT, 2><<<grid, 32 * RM_WARPS, smem, st>>>(c, f, (size_t)g.V * 12, g.V, P, nv, R, Rs);
-  CKL("restrict");
-}
-static void restrict_mma(const FineGeom& g, cplx<float>* c, const void* psi, const float* pn, const __half2* P, int nv, int R, int Rs,
-                         cudaStream_t st) {
-  const Spinor<PREC_F16> f{(__half2*)psi, (float*)pn, g.Vb};
-  if (nv <= 16) restrict_mma_m<1>(g, c, f, P, nv, R, Rs, st);
-  else if (nv <= 32) restrict_mma_m<2>(g, c, f, P, nv, R, Rs, st);
-  else restrict_mma_m<4>(g, c, f, P, nv, R, Rs, st);
-}
-static void prolong_mma(const FineGeom& g, void* x, float* xn, const cplx<float>* e, const __half2* P, int nv, int R, int Rs, int add,
-                        cudaStream_t st) {
-  const size_t smem = (size_t)2 * ((nv + 3) / 4 * 4) * 9 * sizeof(float2);
-  const int threads = g.Vb < 64 ? 2 * g.Vb : 128;  // a warp per 16 sites, four at most
-  k_prolong_mma<<<(unsigned)g.Nb * ((R + 7) / 8), threads, smem, st>>>(Spinor<PREC_F16>{(__half2*)x, xn, g.Vb}, (size_t)g.V * 12,
-                                                                      g.V, e, P, nv, R, Rs, add);
-  CKL("prolong");
-}
-
 void launch_restrict(const FineGeom& g, int pin, cplx<float>* c, const void* psi, const float* pn, const void* P,
                      int pprec, int nv, int R, int Rs, cudaStream_t st) {
   ScopedTimer timer_(pin == PREC_F16 ? "restrict_f16" : pin == PREC_F32 ? "restrict_f32" : "restrict_f64", st, R);
   if (R <= 0) return;
-  if (pprec == PREC_F16 && pin == PREC_F16) restrict_mma(g, c, psi, pn, (const __half2*)P, nv, R, Rs, st);
-  else if (pprec == PREC_F16) restrict_t<__half2>(g, pin, c, psi, pn, (const __half2*)P, nv, R, Rs, st);
+  if (pprec == PREC_F16) restrict_t<__half2>(g, pin, c, psi, pn, (const __half2*)P, nv, R, Rs, st);
   else restrict_t<float2>(g, pin, c, psi, pn, (const float2*)P, nv, R, Rs, st);
 }
 
@@ -874,8 +656,7 @@ void launch_prolong(const FineGeom& g, int pout, void* x, float* xn, const cplx<
                     int nv, int R, int Rs, int add, cudaStream_t st) {
   ScopedTimer timer_(pout == PREC_F16 ? "prolong_f16" : pout == PREC_F32 ? "prolong_f32" : "prolong_f64", st, R);
   if (R <= 0) return;
-  if (pprec == PREC_F16 && pout == PREC_F16) prolong_mma(g, x, xn, e, (const __half2*)P, nv, R, Rs, add, st);
-  else if (pprec == PREC_F16) prolong_t<__half2>(g, pout, x, xn, e, (const __half2*)P, nv, R, Rs, add, st);
+  if (pprec == PREC_F16) prolong_t<__half2>(g, pout, x, xn, e, (const __half2*)P, nv, R, Rs, add, st);
   else prolong_t<float2>(g, pout, x, xn, e, (const float2*)P, nv, R, Rs, add, st);
 }
 
