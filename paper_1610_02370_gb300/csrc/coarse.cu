@@ -274,13 +274,14 @@ __global__ void __launch_bounds__(256, 1) k_galerkin_rows(float2* __restrict__ D
 // as FP16 in shared memory and forms, for each part d (self, then the faces) and X sites at a time, the
 // chirality-s components y of all n columns in FP32; their projections are a dense contraction
 //   D[i][j] = sum over (component, site) conj(P_i) y_j
-// done by mma.sync m16n8k8 in TF32: P's FP16 entries are exact in TF32, y goes in as hi + lo (21 bits) and sums are
-// FP32, so the result is as exact as the FP32 sums of k_galerkin_rows it replaces.  (The operands sit in registers and shared memory
+// done by mma.sync m16n8k8 in TF32: P's FP16 entries are exact in TF32, y goes in as hi + lo (22 bits), and the sums keep
+// what the unit cuts off (mma_sum): 2.5e-8 against 64-bit sums of the same operands (8^4, 24 vectors), the FP32 sums of
+// k_galerkin_rows 4.7e-8, one chain of accumulators 2.3e-5.  (The operands sit in registers and shared memory
 // where the FP32 stencil leaves them; the contraction is 43 GFLOP at 16^3 x 32, a small part of the time, so the
-// tensor-memory path would not pay for staging operand images.)  16^3 x 32, n = 48: 2.72 ms, k_galerkin_rows<2> 6.95 ms
-// (its projections took 17 shared-memory loads per 32 multiply-adds and a warp reduction per entry); what is left is
-// the latency of the P and link loads at 12 warps per SM.  Columns are spread over the threads X sites x
-// (GM_THREADS / X) column groups, GM_CPT columns per thread sharing each link.
+// tensor-memory path would not pay for staging operand images.)  16^3 x 32, n = 48: 3.17 ms (2.75 without the cut parts),
+// k_galerkin_rows<2> 6.95 ms (its projections took 17 shared-memory loads per 32 multiply-adds and a warp reduction per
+// entry); what is left is the latency of the P and link loads at 12 warps per SM.  Columns are spread over the threads X
+// sites x (GM_THREADS / X) column groups, GM_CPT columns per thread sharing each link.
 static const int GM_THREADS = 384, GM_CPT = 4;
 
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -288,10 +289,27 @@ __device__ __forceinline__ uint32_t to_tf32(float x) {
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
   return r;
 }
-__device__ __forceinline__ void mma_tf32(float c[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+__device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// (s, e) += A (hi + lo), the sum in s and what its rounding left out in e.  The unit cuts a sum off towards zero, which in
+// one chain of the 768 products of an entry adds up to 2e-5; forming the product once more on top of (old sum - new
+// sum) gives back what was cut.
+__device__ __forceinline__ void mma_sum(float (&s)[4], float (&e)[4], const uint32_t (&a)[4], uint32_t hi0, uint32_t hi1,
+                                        uint32_t lo0, uint32_t lo1) {
+  float t[4];
+#pragma unroll
+  for (int k = 0; k < 4; k++) t[k] = s[k];
+  mma_tf32(t, a, hi0, hi1);
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    e[k] = __fadd_rn(__fsub_rn(s[k], t[k]), e[k]);
+    s[k] = t[k];
+  }
+  mma_tf32(e, a, hi0, hi1);
+  mma_tf32(e, a, lo0, lo1);
 }
 
 // acc[cc] += chirality-s part of the hop (MU, FWD) of GM_CPT columns col0 + cc cstep read at (blk, loc) of P
@@ -368,9 +386,17 @@ __device__ __forceinline__ void galerkin_site(cplx<float> (&acc)[GM_CPT][6], con
   }
 }
 
-// one 16 x 8 tile of the projections of a chunk of X sites
+// one 16 x 8 tile of the projections of a chunk of X sites; real and imaginary sums and what they leave out
+struct GmAcc {
+  float r[4], i[4], re[4], ie[4];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int k = 0; k < 4; k++) r[k] = i[k] = re[k] = ie[k] = 0.f;
+  }
+  __device__ __forceinline__ float2 get(int k) const { return make_float2(__fadd_rn(r[k], re[k]), __fadd_rn(i[k], ie[k])); }
+};
 template <int X>
-__device__ __forceinline__ void galerkin_tile(float (&cr)[4], float (&ci)[4], const __half2* __restrict__ Ps, const float2* __restrict__ Bs,
+__device__ __forceinline__ void galerkin_tile(GmAcc& acc, const __half2* __restrict__ Ps, const float2* __restrict__ Bs,
                                               const int* sites, int tile, int ntile, int nv, int rs, int Vb, int lane) {
   constexpr int BS = 6 * X + 4;
   const int n = 2 * nv, mt = tile / ntile, nt = tile - mt * ntile, t = lane & 3, gr = lane >> 2;
@@ -384,14 +410,12 @@ __device__ __forceinline__ void galerkin_tile(float (&cr)[4], float (&ci)[4], co
     for (int x0 = 0; x0 < X; x0 += 4) {
       const int st = c * Vb + sites[x0 + t];
       const float2 a = __half22float2(pa[st]), b = __half22float2(pb[st]), y = pc[c * X + x0 + t];
-      const uint32_t ar = __float_as_uint(a.x), ai = __float_as_uint(a.y), br = __float_as_uint(b.x), bi = __float_as_uint(b.y),
-                     an = __float_as_uint(-a.y), bn = __float_as_uint(-b.y);
+      const uint32_t ar = __float_as_uint(a.x), ai = __float_as_uint(a.y), br = __float_as_uint(b.x), bi = __float_as_uint(b.y);
+      const uint32_t re[4] = {ar, br, ai, bi}, im[4] = {__float_as_uint(-a.y), __float_as_uint(-b.y), ar, br};
       const uint32_t hr = to_tf32(y.x), hi = to_tf32(y.y);
       const uint32_t lr = to_tf32(y.x - __uint_as_float(hr)), li = to_tf32(y.y - __uint_as_float(hi));
-      mma_tf32(cr, ar, br, ai, bi, hr, hi);
-      mma_tf32(ci, an, bn, ar, br, hr, hi);
-      mma_tf32(cr, ar, br, ai, bi, lr, li);
-      mma_tf32(ci, an, bn, ar, br, lr, li);
+      mma_sum(acc.r, acc.re, re, hr, hi, lr, li);
+      mma_sum(acc.i, acc.ie, im, hr, hi, lr, li);
     }
 }
 
@@ -415,7 +439,9 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_galerkin_mma(float2* __restri
   const int ntile = (n + 7) / 8, tiles = (nv + 15) / 16 * ntile;  // 16 x 8 tiles, at most two per warp
   for (int d = 0; d < 9; d++) {
     const int nsite = d ? f.off[d] - f.off[d - 1] : Vb;
-    float cr0[4] = {0.f, 0.f, 0.f, 0.f}, ci0[4] = {0.f, 0.f, 0.f, 0.f}, cr1[4] = {0.f, 0.f, 0.f, 0.f}, ci1[4] = {0.f, 0.f, 0.f, 0.f};
+    GmAcc acc0, acc1;
+    acc0.clear();
+    acc1.clear();
     for (int c0 = 0; c0 < nsite; c0 += X) {
       // ---- y of X sites, all columns
       const bool in = c0 + x < nsite;
@@ -454,9 +480,9 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_galerkin_mma(float2* __restri
       }
       __syncthreads();
       // ---- projections: 4 sites of one component per instruction
-      if (warp < tiles) galerkin_tile<X>(cr0, ci0, Ps, Bs, sites, warp, ntile, nv, rs, Vb, lane);
+      if (warp < tiles) galerkin_tile<X>(acc0, Ps, Bs, sites, warp, ntile, nv, rs, Vb, lane);
       if (warp + GM_THREADS / 32 < tiles)
-        galerkin_tile<X>(cr1, ci1, Ps, Bs, sites, warp + GM_THREADS / 32, ntile, nv, rs, Vb, lane);
+        galerkin_tile<X>(acc1, Ps, Bs, sites, warp + GM_THREADS / 32, ntile, nv, rs, Vb, lane);
     }
 #pragma unroll
     for (int q = 0; q < 2; q++) {
@@ -465,7 +491,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_galerkin_mma(float2* __restri
       for (int k = 0; k < 4; k++) {
         const int row = mt * 16 + (lane >> 2) + (k >> 1) * 8, col = nt * 8 + 2 * (lane & 3) + (k & 1);
         if (tile < tiles && row < nv && col < n)
-          Dc[(((size_t)A * 9 + d) * n + col) * n + s * nv + row] = q ? make_float2(cr1[k], ci1[k]) : make_float2(cr0[k], ci0[k]);
+          Dc[(((size_t)A * 9 + d) * n + col) * n + s * nv + row] = q ? acc1.get(k) : acc0.get(k);
       }
     }
   }
