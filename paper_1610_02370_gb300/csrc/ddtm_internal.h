@@ -168,6 +168,7 @@ struct ddtm_ctx {
   ddtm::DevBuf sinv[3];    // per precision, even-site inverse of site term + i mu gamma5
   double sinv_mu[3] = {0, 0, 0};
   bool sinv_ok[3] = {false, false, false};
+  int sap16_op = -1;       // precision of the operator copies that FP16 fields are smoothed with (-1: not decided yet)
   // level-0 aggregation
   int nv0 = 0;
   ddtm::DevBuf tv0;        // test vectors: nv0 fine FP32 fields (internal layout)

@@ -70,21 +70,32 @@ static CoarseLevel& coarsest(ddtm_ctx* c) { return c->p.n_levels == 3 ? c->c2 : 
 static const int ABI_BATCH = 12;
 
 // Operator copies of the smoother for fields of precision prec; returns their precision.  FP16 fields on
-// 4^4 blocks take FP32 copies where the memory for them is there: the block solve reads each entry from L2 many
+// 4^4 blocks take FP32 copies where memory is plentiful: the block solve reads each entry from L2 many
 // times, so halving its bytes gains nothing, while converting it costs as much as a fifth of the kernel
-// (24^3 x 48, 12 right-hand sides, one cycle: 2.70 ms against 3.21 ms with FP16 copies).
+// (24^3 x 48, 12 right-hand sides, one cycle: 2.70 ms against 3.21 ms with FP16 copies).  They add up to 864 B per site to
+// the 432 of the FP16 ones (288 of which ddtm_apply_D_noalloc may still want), so a context decides on its first FP16
+// smoothing, and against them under a memory limit, where a later call may need what they take, and where they would
+// take more than a sixteenth of the free device memory.
 static int sap_operator(ddtm_ctx* c, int prec, double mu) {
   ensure_fine_prec(c, prec);
   if (prec == PREC_F16 && sap_b4_blocks(c->g)) {
-    const bool had_links = c->links[PREC_F32].p, had_clover = c->clover[PREC_F32].p;
-    try {
-      ensure_fine_prec(c, PREC_F32);
-      ensure_site_inverse(c, PREC_F32, mu);
-      return PREC_F32;
-    } catch (const Error& e) {
-      if (e.code != DDTM_ERR_OOM) throw;
-      if (!had_links) c->links[PREC_F32].release();
-      if (!had_clover) c->clover[PREC_F32].release();
+    if (c->sap16_op < 0) {
+      size_t fr = 0, tot = 0;
+      CK(cudaMemGetInfo(&fr, &tot));
+      c->sap16_op = !device_memory_limit() && (size_t)c->g.V * 864 <= fr / 16 ? PREC_F32 : PREC_F16;
+    }
+    if (c->sap16_op == PREC_F32) {
+      const bool had_links = c->links[PREC_F32].p, had_clover = c->clover[PREC_F32].p;
+      try {
+        ensure_fine_prec(c, PREC_F32);
+        ensure_site_inverse(c, PREC_F32, mu);
+        return PREC_F32;
+      } catch (const Error& e) {
+        if (e.code != DDTM_ERR_OOM) throw;
+        if (!had_links) c->links[PREC_F32].release();
+        if (!had_clover) c->clover[PREC_F32].release();
+        c->sap16_op = PREC_F16;
+      }
     }
   }
   ensure_site_inverse(c, prec, mu);
