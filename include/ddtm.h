@@ -331,7 +331,9 @@ int ddtm_autotune_report(char* buf, int len);
  * process (bytes; 0 removes the cap, the default).  An allocation that would
  * exceed it fails with DDTM_ERR_OOM before cudaMalloc is called, exactly as a
  * failed cudaMalloc does; the call that needed it returns DDTM_ERR_OOM and the
- * context stays usable (a later call may succeed under a larger cap).  Lets a
+ * context stays usable (a later call may succeed under a larger cap).  Before
+ * that, workspace that the context keeps only for speed is given back, and
+ * calls fall back to variants that need less memory.  Lets a
  * caller that shares the GPU keep the solver within a share of HBM (the paper
  * has no counterpart; it runs one solver per node). */
 int ddtm_set_memory_limit(size_t bytes);

@@ -16,7 +16,8 @@ using namespace ddtm;
 #define API_BEGIN(ctx)                                   \
   if (!(ctx)) return DDTM_ERR_ARG;                       \
   (ctx)->err.clear();                                    \
-  try {
+  try {                                                  \
+    ddtm::ScratchPool::Scope scope_(&(ctx)->scratch);
 #define API_END(ctx)                                     \
   }                                                      \
   catch (const ddtm::Error& e) {                         \
@@ -87,6 +88,13 @@ void unstage_out(ddtm_ctx* c, double* y, const double* d, size_t ncomplex, int l
   CK(cudaStreamSynchronize(c->stream));
 }
 
+// the staging of one host vector each way, ahead of buffers that the call could do without
+void stage_reserve(ddtm_ctx* c, size_t ncomplex, int loc) {
+  if (loc == DDTM_LOC_DEVICE) return;
+  c->scratch.get("canon_in", ncomplex * 16);
+  c->scratch.get("canon_out", ncomplex * 16);
+}
+
 void field_alloc(ddtm_field* f) {
   size_t V = f->ctx->g.V;
   f->stride = V * 12;
@@ -101,24 +109,25 @@ float* field_nrm(const ddtm_field* f, int r) {
   return f->prec == PREC_F16 ? f->nrm.as<float>() + (size_t)r * f->ctx->g.V : nullptr;
 }
 
-ApiFields::ApiFields(ddtm_ctx* c, int prec, int nrhs, int loc) {
+ApiFields::ApiFields(ddtm_ctx* c, int prec, int nrhs, int loc) : pool(&c->scratch) {
   const size_t V = c->g.V, fb = V * 12 * store2_bytes(prec), nb = prec == PREC_F16 ? V * sizeof(float) : 0;
   const size_t one = (fb + 255) / 256 * 256 + nb;  // per field and right-hand side
+  auto total = [&](int n) { return 2 * ((fb * n + 255) / 256 * 256 + (nb * n + 255) / 256 * 256); };
   batch = 1;
   if (loc == DDTM_LOC_DEVICE)  // host arrays are staged one right-hand side at a time
     while (batch < nrhs && batch < 12 && 2 * one * (batch + 1) <= API_KEEP_BYTES) batch++;
-  const size_t da = (fb * batch + 255) / 256 * 256, tot = 2 * (da + (nb * batch + 255) / 256 * 256);
-  char* p;
-  if (tot <= API_KEEP_BYTES) {
-    p = (char*)c->scratch.get("api_fields", tot);
-  } else {
-    own.ensure(tot);
+  char* p = total(batch) <= API_KEEP_BYTES ? (char*)c->scratch.get_spare("api_fields", total(batch)) : nullptr;
+  if (!p) {
+    batch = 1;
+    own.ensure(total(1));
     p = (char*)own.p;
   }
+  const size_t da = (fb * batch + 255) / 256 * 256;
   a = p;
   b = p + da;
   an = nb ? (float*)(p + 2 * da) : nullptr;
   bn = nb ? (float*)(p + 2 * da + (nb * batch + 255) / 256 * 256) : nullptr;
+  pool->pins++;  // in use from here on
 }
 
 void dslash_field(ddtm_ctx* c, ddtm_field* y, const ddtm_field* x, double mu) {
@@ -325,6 +334,7 @@ int ddtm_apply_D(ddtm_ctx* ctx, double* y, const double* x, int nrhs, double mu,
   if (nrhs == 0) return DDTM_OK;
   ensure_fine_prec(ctx, prec);
   size_t nsp = (size_t)ctx->g.V * 12;
+  stage_reserve(ctx, nsp, loc);
   ApiFields f(ctx, prec, nrhs, loc);
   for (int r = 0; r < nrhs; r += f.batch) {
     const int R = nrhs - r < f.batch ? nrhs - r : f.batch;

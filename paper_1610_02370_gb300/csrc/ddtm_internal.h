@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <map>
+#include <set>
 #include <stdexcept>
 #include <string>
 #include <vector>
@@ -136,10 +137,33 @@ struct CoefRing {
   const double2* push(const double2* vals, size_t count, cudaStream_t st);
 };
 
+// Named work buffers of a context, kept from call to call.  Spare ones are those that a call can do without, because it has
+// a variant that needs less memory: they are given back when an allocation of their context finds no room, unless
+// the running call uses them (Pin).
 struct ScratchPool {
   std::map<std::string, DevBuf*> bufs;
+  std::set<std::string> spare;
+  int pins = 0;
+  struct Pin {
+    ScratchPool* p;
+    explicit Pin(ScratchPool* q) : p(q) { p->pins++; }
+    Pin(const Pin&) = delete;
+    Pin& operator=(const Pin&) = delete;
+    ~Pin() { p->pins--; }
+  };
+  // the pool whose spare buffers this thread's allocations may reclaim: that of the context of the running call
+  struct Scope {
+    ScratchPool* saved;
+    explicit Scope(ScratchPool* p);
+    Scope(const Scope&) = delete;
+    Scope& operator=(const Scope&) = delete;
+    ~Scope();
+  };
   ~ScratchPool();
   void* get(const std::string& name, size_t bytes);
+  void* get_spare(const std::string& name, size_t bytes);  // null (and nothing held by that name) where there is no room
+  void drop(const std::string& name);                      // frees one buffer
+  bool reclaim();                                          // frees the spare buffers; true if that freed anything
   void clear();                                       // frees every buffer
   size_t held(const std::string& prefix) const;  // bytes held by buffers whose name starts with prefix
 };
@@ -209,14 +233,19 @@ namespace ddtm {
 // Two internal fields of precision prec for a call on canonical spinors, `batch` right-hand sides at once (as many
 // as fit API_KEEP_BYTES for device arrays, one for host arrays).  Up to API_KEEP_BYTES they are kept with
 // the context's scratch (allocating and freeing them costs 0.1 ms per call, as much as the call itself on a small
-// lattice); larger ones live as long as the object.
+// lattice) as a spare buffer; larger ones, and those of one right-hand side that a call makes do with where memory is
+// short, live as long as the object.
 static const size_t API_KEEP_BYTES = (size_t)64 << 20;
 struct ApiFields {
+  ScratchPool* pool;
   int batch;
   void *a, *b;
   float *an, *bn;
   DevBuf own;
   ApiFields(ddtm_ctx* c, int prec, int nrhs, int loc);
+  ~ApiFields() { pool->pins--; }
+  ApiFields(const ApiFields&) = delete;
+  ApiFields& operator=(const ApiFields&) = delete;
 };
 
 // ---- geometry.cu -------------------------------------------------------------

@@ -267,6 +267,7 @@ extern "C" int ddtm_eo_cg(ddtm_ctx* ctx, double* x, const double* b, int nrhs, d
   if (!ctx) return DDTM_ERR_ARG;
   ctx->err.clear();
   try {
+    ScratchPool::Scope scope_(&ctx->scratch);
     check_loc(loc);
     if (!x || !b || nrhs < 0 || !std::isfinite(mu) || !(tol > 0) || max_iter < 0)
       throw Error(DDTM_ERR_ARG, "invalid arguments");

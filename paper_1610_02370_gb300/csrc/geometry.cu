@@ -65,19 +65,23 @@ void DevBuf::release() {
   bytes = 0;
 }
 
+static thread_local ScratchPool* t_pool = nullptr;  // see ScratchPool::Scope
+
 void DevBuf::ensure(size_t n) {
   if (n <= bytes && p) return;
   release();
   if (n == 0) return;
-  const size_t lim = g_dev_limit.load();
-  if (lim && g_dev_bytes.load() + n > lim)
-    throw Error(DDTM_ERR_OOM, "device allocation of " + std::to_string(n) + " bytes would exceed the library's "
-                                  "memory limit of " + std::to_string(lim) + " bytes (" +
-                                  std::to_string(g_dev_bytes.load()) + " in use)");
-  cudaError_t e = cudaMalloc(&p, n);
-  if (e != cudaSuccess) {
+  while (true) {  // until there is room, or nothing left to give back
+    const size_t lim = g_dev_limit.load();
+    const bool over = lim && g_dev_bytes.load() + n > lim;
+    if (!over && cudaMalloc(&p, n) == cudaSuccess) break;
     p = nullptr;
-    cudaGetLastError();
+    if (!over) cudaGetLastError();
+    if (t_pool && t_pool->reclaim()) continue;
+    if (over)
+      throw Error(DDTM_ERR_OOM, "device allocation of " + std::to_string(n) + " bytes would exceed the library's "
+                                    "memory limit of " + std::to_string(lim) + " bytes (" +
+                                    std::to_string(g_dev_bytes.load()) + " in use)");
     throw Error(DDTM_ERR_OOM, "device allocation of " + std::to_string(n) + " bytes failed");
   }
   bytes = n;
@@ -104,6 +108,39 @@ void* ScratchPool::get(const std::string& name, size_t bytes) {
   b->ensure(bytes < 256 ? 256 : bytes);
   return b->p;
 }
+
+void* ScratchPool::get_spare(const std::string& name, size_t bytes) {
+  spare.insert(name);
+  try {
+    return get(name, bytes);
+  } catch (const Error& e) {
+    if (e.code != DDTM_ERR_OOM) throw;
+  }
+  drop(name);
+  return nullptr;
+}
+
+void ScratchPool::drop(const std::string& name) {
+  auto it = bufs.find(name);
+  if (it == bufs.end()) return;
+  delete it->second;
+  bufs.erase(it);
+}
+
+bool ScratchPool::reclaim() {
+  bool freed = false;
+  if (pins == 0)
+    for (const auto& name : spare) {
+      auto it = bufs.find(name);
+      if (it == bufs.end() || !it->second->p) continue;
+      it->second->release();
+      freed = true;
+    }
+  return freed;
+}
+
+ScratchPool::Scope::Scope(ScratchPool* p) : saved(t_pool) { t_pool = p; }
+ScratchPool::Scope::~Scope() { t_pool = saved; }
 
 size_t ScratchPool::held(const std::string& prefix) const {
   size_t s = 0;

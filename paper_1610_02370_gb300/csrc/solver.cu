@@ -11,6 +11,7 @@
 #include <chrono>
 #include <complex>
 #include <functional>
+#include <memory>
 
 #include "blas.h"
 #include "coarse.h"
@@ -437,17 +438,56 @@ static int gmres_b(ddtm_ctx* c, const OpF32& A, cplx<float>* x, const cplx<float
 // kernel.  A(w, image, xs, xs_type): w = A v for the FP16 image of v, xs the same v for the twist.
 typedef std::function<void(float*, const void*, const void*, int)> OpImg;
 
-static int gmres_img(ddtm_ctx* c, CoarseLevel& L, const ImgVec& v, int ctas, const OpImg& A, float* x, const float* b, int m,
+// Buffers of a solve with up to m basis vectors, ctas CTAs per step: the basis, the new vector, an image of x, the Krylov
+// scalars, partial sums, and the right-hand side and solution in image order.  All of them are spare (gmres_b needs
+// less where dofs or right-hand sides are padded) and pinned while this lives; ok is false, and none is held, where
+// there is no memory for them.
+struct ImgBuffers {
+  ScratchPool::Pin pin;
+  void* p[7];
+  bool ok = true;
+  char* V() const { return (char*)p[0]; }
+  float* w() const { return (float*)p[1]; }
+  char* xh() const { return (char*)p[2]; }
+  double2* state() const { return (double2*)p[3]; }
+  char* part() const { return (char*)p[4]; }
+  float* b() const { return (float*)p[5]; }
+  float* x() const { return (float*)p[6]; }
+  ImgBuffers(ddtm_ctx* c, const ImgVec& v, int m, int ctas) : pin(&c->scratch) {
+    ScratchPool* pool = &c->scratch;
+    const size_t vb = v.entries() * sizeof(__half), fb = v.entries() * sizeof(float), R = v.t.R;
+    const std::pair<const char*, size_t> bufs[7] = {
+        {"cgi_V", (size_t)(m + 1) * vb},
+        {"cgi_w", fb},
+        {"cgi_xh", vb},
+        {"cgi_state", (R * (m + 1) * m + 2 * R * m + R * (m + 1) + 2 * (m + 1) * R) * sizeof(double2) + 2 * R * sizeof(double)},
+        {"cgi_part", (size_t)m * R * ctas * sizeof(float2) + R * ctas * sizeof(double) + 64},
+        {"ceo_bi", fb},
+        {"ceo_xi", fb}};
+    if (const size_t lim = device_memory_limit()) {  // known beforehand: no allocation that is taken back in every call
+      size_t in_use = device_bytes_in_use();
+      for (const auto& d : bufs) {
+        const size_t held = pool->held(d.first);
+        if (d.second > held) in_use += d.second - held;
+      }
+      ok = in_use <= lim;
+    }
+    for (int k = 0; ok && k < 7; k++) ok = (p[k] = pool->get_spare(bufs[k].first, bufs[k].second)) != nullptr;
+    if (!ok)
+      for (const auto& d : bufs) pool->drop(d.first);
+  }
+};
+static int gmres_img(ddtm_ctx* c, CoarseLevel& L, const ImgVec& v, int ctas, const ImgBuffers& buf, const OpImg& A, int m,
                      int max_restarts, double tol, double* relres, const std::string& op_key) {
   const int R = v.t.R;
   const size_t ne = v.entries(), vb = ne * sizeof(__half);
-  char* V = (char*)c->scratch.get("cgi_V", (size_t)(m + 1) * vb);
-  float* w = (float*)c->scratch.get("cgi_w", ne * sizeof(float));
-  char* xh = (char*)c->scratch.get("cgi_xh", vb);
+  char *V = buf.V(), *xh = buf.xh();
+  float *w = buf.w(), *x = buf.x();
+  const float* b = buf.b();
   auto Vj = [&](int j) { return (void*)(V + (size_t)j * vb); };
   GsBuffers gb;
   const size_t nH = (size_t)R * (m + 1) * m, ncs = (size_t)R * m, ng = (size_t)R * (m + 1), nh = (size_t)(m + 1) * R;
-  double2* st2 = (double2*)c->scratch.get("cgi_state", (nH + 2 * ncs + ng + 2 * nh) * sizeof(double2) + 2 * (size_t)R * sizeof(double));
+  double2* st2 = buf.state();
   ArnoldiDev ad;
   ad.H = st2;
   ad.cs = ad.H + nH;
@@ -460,8 +500,7 @@ static int gmres_img(ddtm_ctx* c, CoarseLevel& L, const ImgVec& v, int ctas, con
   ad.est = ad.bn + R;
   ad.m = m;
   ad.R = R;
-  char* pb = (char*)c->scratch.get("cgi_part", (size_t)m * R * ctas * sizeof(float2) + (size_t)R * ctas * sizeof(double) + 64);
-  gb.part = (float2*)pb;
+  gb.part = (float2*)buf.part();
   gb.npart = (double*)(gb.part + (size_t)m * R * ctas);
   gb.bar = (unsigned*)(gb.npart + (size_t)R * ctas);
   gb.err = L.tc_err.as<int>();
@@ -581,23 +620,25 @@ int coarse_eo_solve(ddtm_ctx* c, cplx<float>* x_full, const cplx<float>* b_full,
   snprintf(ok, sizeof(ok), "eo|mu%.17g|n%d|p%d|lev%p", mu_c, L.n, L.prec, (const void*)&L);
   const ImgVec v{tc_geom(L.n, Rc), (int)no};
   const int ctas = L.prec == PREC_F16 && tol >= 1e-3 ? gs_ctas(v, restart) : 0;
-  if (ctas > 0) {
+  char* tt = L.prec == PREC_F16 ? (char*)c->scratch.get("ceo_tt", tc_vector_image_bytes(L, (int)ne, Rc)) : nullptr;
+  std::unique_ptr<ImgBuffers> img;
+  if (ctas > 0) img.reset(new ImgBuffers(c, v, restart, ctas));
+  if (img && !img->ok) img.reset();
+  if (img) {
     // tensor cores on image-ordered vectors; tighter tolerances need the second Gram-Schmidt pass of gmres_b
-    char* tt = (char*)c->scratch.get("ceo_tt", tc_vector_image_bytes(L, (int)ne, Rc));
-    float* bi = (float*)c->scratch.get("ceo_bi", v.entries() * sizeof(float));
-    float* xi = (float*)c->scratch.get("ceo_xi", v.entries() * sizeof(float));
+    float *bi = img->b(), *xi = img->x();
     launch_img_order(v, bi, bo, 0, c->stream);
-    OpImg Dimg = [&, tt](float* out, const void* img, const void* xs, int xs_type) {
-      TcPass h = hop_even_pass(L, img, tt);
+    OpImg Dimg = [&, tt](float* out, const void* vin, const void* xs, int xs_type) {
+      TcPass h = hop_even_pass(L, vin, tt);
       launch_coarse_tc(L, h, Rc, c->stream);
-      TcPass o = odd_pass(L, img, tt, mu_c);
+      TcPass o = odd_pass(L, vin, tt, mu_c);
       o.y = reinterpret_cast<cplx<float>*>(out);
       o.y_img = true;
       o.xs = xs;
       o.xs_type = xs_type;
       launch_coarse_tc(L, o, Rc, c->stream);
     };
-    const int it = gmres_img(c, L, v, ctas, Dimg, xi, bi, restart, max_restarts, tol, relres, std::string(ok));
+    const int it = gmres_img(c, L, v, ctas, *img, Dimg, restart, max_restarts, tol, relres, std::string(ok));
     launch_img_order(v, xi, xo, 1, c->stream);
     launch_coarse_even(L, te, be, xo, Rc, 1.f, -1.f, c->stream);  // phi_e = D_ee^-1 (eta_e - D_eo phi_o)
     launch_parity_copy(L, 0, te, x_full, Rc, 1, c->stream);
@@ -609,9 +650,7 @@ int coarse_eo_solve(ddtm_ctx* c, cplx<float>* x_full, const cplx<float>* b_full,
   if (L.prec == PREC_F16) {
     // tensor cores: FP16 images of the operand vectors, FP32 accumulation;
     // only the input and the output of D_hat are FP32 vectors
-    const size_t img_o = tc_vector_image_bytes(L, (int)no, Rc), img_e = tc_vector_image_bytes(L, (int)ne, Rc);
-    char* vt = (char*)c->scratch.get("ceo_vt", img_o);
-    char* tt = (char*)c->scratch.get("ceo_tt", img_e);
+    char* vt = (char*)c->scratch.get("ceo_vt", tc_vector_image_bytes(L, (int)no, Rc));
     Dhat = [&, vt, tt](cplx<float>* out, const void* in, int in_type) {
       launch_vector_image(L, vt, in, in_type, (int)no, Rc, c->stream);
       launch_coarse_tc(L, hop_even_pass(L, vt, tt), Rc, c->stream);
@@ -1004,7 +1043,8 @@ void run_setup(ddtm_ctx* c, double mu, uint64_t seed, bool update = false, int n
 #define API_BEGIN(ctx)             \
   if (!(ctx)) return DDTM_ERR_ARG; \
   (ctx)->err.clear();              \
-  try {
+  try {                            \
+    ddtm::ScratchPool::Scope scope_(&(ctx)->scratch);
 #define API_END(ctx)                \
   }                                 \
   catch (const ddtm::Error& e) {    \
@@ -1072,8 +1112,9 @@ int ddtm_sap(ddtm_ctx* ctx, double* x, const double* b, int nrhs, double mu, int
   check_loc(loc);
   if (!x || !b || nrhs < 0 || ncycles < 0 || nmr < 0) throw Error(DDTM_ERR_ARG, "invalid arguments");
   if (nrhs == 0) return DDTM_OK;
-  ensure_fine_prec(ctx, prec);
+  sap_operator(ctx, prec, mu);
   size_t nsp = (size_t)ctx->g.V * 12;
+  stage_reserve(ctx, nsp, loc);
   ApiFields f(ctx, prec, nrhs, loc);
   for (int r = 0; r < nrhs; r += f.batch) {
     const int R = nrhs - r < f.batch ? nrhs - r : f.batch;
@@ -1330,22 +1371,26 @@ int ddtm_apply_Dc(ddtm_ctx* ctx, int level, double* y, const double* x, int nrhs
   const bool apart = y + 2 * nc * nrhs <= x || x + 2 * nc * nrhs <= y;
   if (L.prec == PREC_F16 && loc == DDTM_LOC_DEVICE && apart) {
     // canonical vectors to operand images and back in one launch each, image-ordered FP32 between (12 vectors of
-    // 32^3 x 64: 56 us for both, through interleaved batches 72 and a batch more in memory)
+    // 32^3 x 64: 56 us for both, through interleaved batches 72), where there is memory for the padded right-hand sides
     const ImgVec v{tc_geom(L.n, nrhs), L.Nc};
     char* xt = (char*)ctx->scratch.get("abi_ct", tc_vector_image_bytes(L, L.Nc, nrhs));
-    float* xi = (float*)ctx->scratch.get("abi_ci", v.entries() * sizeof(float));
-    float* yi = (float*)ctx->scratch.get("abi_cib", v.entries() * sizeof(float));
-    launch_img_from_canon(v, xt, xi, x, ctx->stream);
-    TcPass f = full_pass(L, xt, mu);
-    f.y = reinterpret_cast<cplx<float>*>(yi);
-    f.y_img = true;
-    f.xs = xi;
-    f.xs_type = 4;
-    launch_coarse_tc(L, f, nrhs, ctx->stream);
-    launch_img_to_canon(v, y, yi, ctx->stream);
-    CK(cudaStreamSynchronize(ctx->stream));
-    check_tc_error(L);
-    return DDTM_OK;
+    ScratchPool::Pin pin(&ctx->scratch);
+    float* xi = (float*)ctx->scratch.get_spare("abi_ci", v.entries() * sizeof(float));
+    float* yi = xi ? (float*)ctx->scratch.get_spare("abi_cib", v.entries() * sizeof(float)) : nullptr;
+    if (yi) {
+      launch_img_from_canon(v, xt, xi, x, ctx->stream);
+      TcPass f = full_pass(L, xt, mu);
+      f.y = reinterpret_cast<cplx<float>*>(yi);
+      f.y_img = true;
+      f.xs = xi;
+      f.xs_type = 4;
+      launch_coarse_tc(L, f, nrhs, ctx->stream);
+      launch_img_to_canon(v, y, yi, ctx->stream);
+      CK(cudaStreamSynchronize(ctx->stream));
+      check_tc_error(L);
+      return DDTM_OK;
+    }
+    ctx->scratch.drop("abi_ci");
   }
   // all right-hand sides go through one batched stencil pass
   cplx<float>* xv = (cplx<float>*)ctx->scratch.get("abi_c32", nc * nrhs * 8);

@@ -18,6 +18,7 @@ void ensure_fine_prec(ddtm_ctx* c, int prec);
 void ensure_site_inverse(ddtm_ctx* c, int prec, double mu);
 const double* stage_in(ddtm_ctx* c, const char* name, const double* x, size_t ncomplex, int loc);
 double* stage_out(ddtm_ctx* c, const char* name, double* y, size_t ncomplex, int loc);
+void stage_reserve(ddtm_ctx* c, size_t ncomplex, int loc);
 void unstage_out(ddtm_ctx* c, double* y, const double* d, size_t ncomplex, int loc);
 void field_alloc(ddtm_field* f);
 void* field_ptr(const ddtm_field* f, int r);

@@ -84,3 +84,82 @@ def test_setup_and_solve_fit_in_what_they_need(lib):
             lib.ddtm_set_memory_limit(0)
             lib.ddtm_destroy(ctx)
     assert used[1] <= used[0] - V * 144 + SLACK
+
+
+@pytest.mark.parametrize("loc", ["cuda", "cpu"])
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_canonical_calls_of_many_vectors(lib, ctx, prec, loc):
+    """Operator copies, two fields of one right-hand side, and host arrays staged one vector each way: that is enough for
+    twelve right-hand sides, and the same bits as without a limit."""
+    one = {0: 192, 1: 96, 2: 52}[prec]
+    b = synth.gaussian_spinor(DIMS, seed=104, nrhs=12, device=loc)
+    want = []
+    for limited in (False, True):
+        for f in (lambda y: lib.ddtm_apply_D(ctx, y, b, 12, 0.003, prec),
+                  lambda y: lib.ddtm_sap(ctx, y, b, 12, 0.003, 2, 3, prec)):
+            y = torch.zeros_like(b)
+            if limited:  # the operator copies are there from the calls before
+                limit(lib, V * (2 * one + (2 * 192 if loc == "cpu" else 0)))
+            f(y)
+            torch.cuda.synchronize()
+            lib.ddtm_set_memory_limit(0)
+            want.append(y)
+        lib.ddtm_release_workspace(ctx)
+    assert torch.equal(want[0], want[2]) and torch.equal(want[1], want[3])
+
+
+def hierarchy(lib, ctx, nv):
+    p = lib.ddtm_get_params(ctx)
+    p.nv[0], p.coarse_prec, p.coarse_tol = nv, lib.PREC_F16, 1e-2
+    lib.ddtm_set_params(ctx, p)
+    lat = (DIMS[0], DIMS[3], DIMS[2], DIMS[1])
+    lib.ddtm_set_test_vectors(ctx, 0, synth.gaussian_vectors((nv,) + lat + (4, 3), seed=105, device="cuda"), nv)
+    return p, synth.gaussian_vectors((1,) + tuple(n // 4 for n in lat) + (2 * nv,), seed=106, device="cuda")
+
+
+def test_coarse_calls_of_one_vector(lib, ctx):
+    """The FP16 operand image (8 columns of 48 padded dofs), two interleaved batches of one column, and for the solve the
+    basis of one column: image order pads the vectors to four columns."""
+    nv = 20
+    n, Nc, m = 2 * nv, V // 256, 100
+    p, b = hierarchy(lib, ctx, nv)
+    want, x = torch.zeros_like(b), torch.zeros_like(b)
+    lib.ddtm_apply_Dc(ctx, 1, want, b, 1, 0.02)
+    p.coarse_restart = 1
+    lib.ddtm_set_params(ctx, p)
+    lib.ddtm_coarse_solve(ctx, x, b, 0.02)  # the inverses of the even sites belong to the operator
+    p.coarse_restart = m
+    lib.ddtm_set_params(ctx, p)
+    lib.ddtm_release_workspace(ctx)
+
+    image = Nc * 8 * 48 * 2
+    limit(lib, image + 2 * Nc * n * 8)
+    y = torch.zeros_like(b)
+    lib.ddtm_apply_Dc(ctx, 1, y, b, 1, 0.02)
+    assert torch.equal(y, want)
+    lib.ddtm_set_memory_limit(0)
+    lib.ddtm_release_workspace(ctx)
+
+    # basis in FP16, eleven batches on half of the sites or their equivalent, both images, Krylov scalars
+    limit(lib, (m + 1) * Nc // 2 * n * 4 + 11 * Nc // 2 * n * 8 + image + (m + 1) * (m + 8) * 16 + (1 << 20))
+    iters, code = lib.ddtm_coarse_solve(ctx, x, b, 0.02)
+    assert code == lib.OK and iters > 0
+    lib.ddtm_set_memory_limit(0)
+    lib.ddtm_apply_Dc(ctx, 1, y, x, 1, 0.02)
+    assert float((b - y).norm() / b.norm()) < 2e-2 + 3e-3
+
+
+def test_spare_buffers_make_room(lib, ctx):
+    """What a coarse solve keeps only for speed is given back when another call needs the memory, and taken again later."""
+    p, b = hierarchy(lib, ctx, 24)
+    x, x2 = torch.zeros_like(b), torch.zeros_like(b)
+    iters, code = lib.ddtm_coarse_solve(ctx, x, b, 0.02)
+    assert code == lib.OK
+    basis = 101 * (V // 512) * 8 * 48 * 2
+    nrhs = basis // (V * 192) + 1  # the fields take more than the free room, and less than that and the basis
+    limit(lib, nrhs * V * 192 - basis // 2)
+    f = lib.ddtm_field_create(ctx, lib.PREC_F64, nrhs)
+    lib.ddtm_field_destroy(f)
+    lib.ddtm_set_memory_limit(0)
+    assert lib.ddtm_coarse_solve(ctx, x2, b, 0.02) == (iters, code)
+    assert torch.equal(x, x2)
