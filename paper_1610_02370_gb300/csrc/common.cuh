@@ -129,6 +129,16 @@ __device__ __forceinline__ Nbr neighbour(const Geo& g, int blk, int loc, int k) 
   return n;
 }
 
+// 1 / sqrt(x) in FP64 from the FP32 estimate by three Newton steps (y += y (1 - x y^2) / 2): a third of the dependent
+// FP64 operations of sqrt and a division, whose latency is long on this GPU.  x > 0 is a sum of FP32 squares.
+__device__ __forceinline__ double inv_sqrt(double x) {
+  if (x < 1e-30 || x > 1e30) return 1.0 / sqrt(x);  // outside the estimate's range
+  double y = (double)rsqrtf((float)x);
+#pragma unroll
+  for (int k = 0; k < 3; k++) y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  return y;
+}
+
 // ---- field views -----------------------------------------------------------
 template <int P>
 struct Spinor {

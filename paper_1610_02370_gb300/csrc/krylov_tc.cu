@@ -162,15 +162,6 @@ __device__ void givens_turn(const GsArgs& a, int r, cplx<float>* s, int lane) {
   double2* H = a.a.H + (size_t)r * (m + 1) * m;
   for (int i = lane; i < j; i += 32) H[(size_t)i * m + j] = make_double2((double)col[i].re, (double)col[i].im);
 }
-// 1 / sqrt(x) in FP64 from the FP32 estimate by three Newton steps (y += y (1 - x y^2) / 2): a third of the dependent
-// FP64 operations of sqrt and a division, whose latency is long on this GPU.  x > 0 is a sum of FP32 squares.
-__device__ __forceinline__ double inv_sqrt(double x) {
-  if (x < 1e-30 || x > 1e30) return 1.0 / sqrt(x);  // outside the estimate's range
-  double y = (double)rsqrtf((float)x);
-#pragma unroll
-  for (int k = 0; k < 3; k++) y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
-  return y;
-}
 // The new rotation, once the norm is known: one thread.  inv_n: 1 / norm (0 if it vanished)
 __device__ void givens_close(const GsArgs& a, int r, double nr2, double inv_n, const cplx<float>* col) {
   const int j = a.nvec - 1, m = a.a.m;
@@ -613,6 +604,7 @@ void launch_img_combine(const ImgVec& v, float* x, const void* V, size_t ldv, in
   if (nvec <= 0) return;
   const int kg4 = 4 * (v.t.kpad / 8);
   const size_t items = (size_t)v.nsites * v.t.ngj * kg4, smem = (size_t)nvec * v.t.R * sizeof(float2);
+  if (smem > 200 * 1024) throw Error(DDTM_ERR_ARG, "internal: coefficient block too large");
   set_dynamic_smem((const void*)k_img_combine, smem);
   size_t grid = (items + 255) / 256;
   if (grid > 4096) grid = 4096;

@@ -4,6 +4,7 @@
 #include "coarse.h"
 #include "common.cuh"
 #include "ddtm_internal.h"
+#include "krylov_tc.h"
 
 using namespace ddtm;
 
@@ -23,7 +24,25 @@ static void set_geom(FineGeom& g, int Vb, int Nb) {
   g.V = (long)Vb * Nb;
 }
 
+__global__ void k_inv_sqrt(const double* x, double* y, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = inv_sqrt(x[i]);
+}
+
 extern "C" {
+int ik_inv_sqrt(const double* x, double* y, int n) {
+  return run([&] {
+    k_inv_sqrt<<<(n + 127) / 128, 128>>>(x, y, n);
+    CKL("inv_sqrt");
+  });
+}
+// x += sum_i y[i R + r] V_i on image-ordered vectors of R right-hand sides, n dofs and nsites sites
+int ik_img_combine(float* x, const void* V, int nvec, const double* y, int n, int R, int nsites) {
+  return run([&] {
+    const ImgVec v{tc_geom(n, R), nsites};
+    launch_img_combine(v, x, V, v.entries() * sizeof(__half), nvec, (const double2*)y, 0);
+  });
+}
 // FP16 fields (complex half [r][block][12][Vb], one scale per site) and FP16 P ([block][2][nv][6][Vb]); the coarse side is
 // complex FP32, column r of Rs
 int ik_restrict(int Vb, int Nb, void* c, const void* psi, const float* pn, const void* P, int nv, int R, int Rs) {
