@@ -530,9 +530,12 @@ void launch_galerkin(const FineGeom& g, const FaceDev& faces, int dprec, void* D
   Clover<PREC_F32> C{(const float2*)clover32, g.Vb};
   if (dprec != PREC_F32) throw Error(DDTM_ERR_ARG, "internal: Galerkin output is FP32");
   const size_t srows1 = galerkin_rows_smem(g, faces, nv, 1), srows2 = galerkin_rows_smem(g, faces, nv, 2);
-  // matrix instructions with the widest chunk whose rows and columns fit in shared memory
-  if (rows_fp16 && (try_galerkin_mma<32>(g, (float2*)Dc, P, U, C, q, f, nv, st) || try_galerkin_mma<16>(g, (float2*)Dc, P, U, C, q, f, nv, st) ||
-                    try_galerkin_mma<8>(g, (float2*)Dc, P, U, C, q, f, nv, st))) {
+  // FP16 rows of P where FP16 coarse storage is asked for and they fit in shared memory with the columns of k_galerkin_rows
+  // (4^4 aggregates: up to 30 vectors); beyond that the rows stay FP32 (k_galerkin), although the matrix instructions
+  // would hold two vectors more: FP16 rows there cost D_c another 2e-4.  Widest chunk of sites that fits.
+  const bool rows = rows_fp16 && (srows1 <= 220 * 1024 || srows2 <= 224 * 1024);
+  if (rows && (try_galerkin_mma<32>(g, (float2*)Dc, P, U, C, q, f, nv, st) || try_galerkin_mma<16>(g, (float2*)Dc, P, U, C, q, f, nv, st) ||
+               try_galerkin_mma<8>(g, (float2*)Dc, P, U, C, q, f, nv, st))) {
   } else if (rows_fp16 && srows2 <= 224 * 1024) {  // two columns per pass where the shared memory holds them
     set_dynamic_smem((const void*)k_galerkin_rows<2>, srows2);
     k_galerkin_rows<2><<<g.Nb * 2, threads, srows2, st>>>((float2*)Dc, P, U, C, q, f, nv);
