@@ -134,154 +134,19 @@ __global__ void k_galerkin(DS* __restrict__ Dc, const float2* __restrict__ P, Li
   }
 }
 
-// The same Galerkin products with the rows staged in shared memory, for FP16
-// coarse storage (the tensor-core images round D_c to FP16 anyway): one CTA
-// per (aggregate A, row chirality s) keeps the nv rows (s, i) of P on A as
-// FP16 in shared memory, computes for CC columns (s', j) at a time the
-// chirality-s components of y_0 and of the face hops y_k as above (each link
-// loaded once for the CC columns), and projects them out of shared memory, each
-// row entry loaded once for the CC columns, so P is not re-read from memory
-// for every column and the projections need fewer shared-memory loads per
-// multiply-add.  Every entry is the same sum, in the same order, for any CC.
-template <int CC>
-__global__ void __launch_bounds__(256, 1) k_galerkin_rows(float2* __restrict__ Dc, const float2* __restrict__ P,
-                                                          Links<PREC_F32> U, Clover<PREC_F32> C, Geo g, FaceTables f,
-                                                          int nv) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int Vb = g.Vb, nf = f.off[8];
-  const int A = blockIdx.x >> 1, s = blockIdx.x & 1;
-  const int n = 2 * nv;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __half2* Ps = reinterpret_cast<__half2*>(smem_raw);                                // [nv][6][Vb]
-  cplx<float>* y0 = reinterpret_cast<cplx<float>*>(Ps + (size_t)nv * 6 * Vb);          // [CC][6][Vb]
-  cplx<float>* yf = y0 + (size_t)CC * 6 * Vb;                                          // [CC][6][nf]
-  const size_t rows0 = pix(A, s, 0, 0, 0, nv, Vb);
-  for (int e = threadIdx.x; e < nv * 6 * Vb; e += blockDim.x) Ps[e] = __float22half2_rn(__ldg(P + rows0 + e));
-  for (int col0 = 0; col0 < n; col0 += CC) {
-    const int ncol = n - col0 < CC ? n - col0 : CC;
-    for (int loc = threadIdx.x; loc < Vb; loc += blockDim.x) {
-      cplx<float> acc[CC][12];
-#pragma unroll
-      for (int cc = 0; cc < CC; cc++)
-#pragma unroll
-        for (int c = 0; c < 12; c++) acc[cc][c] = cplx<float>(0, 0);
-      for (int k = 0; k < 8; k++) {
-        const int mu = k >> 1;
-        const bool fwd = (k & 1) == 0;
-        Nbr nb = neighbour(g, A, loc, k);
-        cplx<float> u[9];
-        if (fwd) U.load(A, loc, mu, u);
-        else U.load(nb.blk, nb.loc, mu, u);
-        const int slot = nb.cross ? f.off[k] + f.idx[k * Vb + loc] : 0;
-#pragma unroll
-        for (int cc = 0; cc < CC; cc++) {
-          if (cc >= ncol) break;
-          const int col = col0 + cc, sp = col / nv, j = col - sp * nv;
-          cplx<float> p[12], h[6], wv[6];
-#pragma unroll
-          for (int c = 0; c < 12; c++)  // column (sp, j): chirality-sp components only (static indices)
-            p[c] = (c / 6 == sp) ? ld(P + pix(nb.blk, sp, j, c % 6, nb.loc, nv, Vb)) : cplx<float>(0, 0);
-          project<float>(mu, fwd, p, h);
-          if (fwd) mul_U<float>(u, h, wv);
-          else mul_Udag<float>(u, h, wv);
-          if (nb.flip)
-            for (int q = 0; q < 6; q++) wv[q] = -wv[q];
-          if (!nb.cross) {
-            reconstruct<float>(mu, fwd, wv, acc[cc]);
-          } else {
-            cplx<float> part[12];
-#pragma unroll
-            for (int c = 0; c < 12; c++) part[c] = cplx<float>(0, 0);
-            reconstruct<float>(mu, fwd, wv, part);
-#pragma unroll
-            for (int c = 0; c < 6; c++) yf[((size_t)cc * 6 + c) * nf + slot] = -0.5f * (s ? part[6 + c] : part[c]);
-          }
-        }
-      }
-#pragma unroll
-      for (int cc = 0; cc < CC; cc++) {
-        if (cc >= ncol) break;
-        const int col = col0 + cc, sp = col / nv, j = col - sp * nv;
-        cplx<float> phi[12], out[12];
-#pragma unroll
-        for (int c = 0; c < 12; c++)
-          phi[c] = (c / 6 == sp) ? ld(P + pix(A, sp, j, c % 6, loc, nv, Vb)) : cplx<float>(0, 0);
-        C.apply(A, loc, phi, out);
-#pragma unroll
-        for (int c = 0; c < 6; c++)
-          y0[((size_t)cc * 6 + c) * Vb + loc] = s ? out[6 + c] + (-0.5f) * acc[cc][6 + c] : out[c] + (-0.5f) * acc[cc][c];
-      }
-    }
-    __syncthreads();
-    const int GR = 4, ngr = (nv + GR - 1) / GR;
-    for (int o = w; o < 9 * ngr; o += nw) {
-      const int d = o / ngr, r0 = (o - d * ngr) * GR;
-      cplx<float> acc[GR][CC];
-      int ir[GR];
-#pragma unroll
-      for (int r = 0; r < GR; r++) {
-#pragma unroll
-        for (int cc = 0; cc < CC; cc++) acc[r][cc] = cplx<float>(0, 0);
-        ir[r] = r0 + r < nv ? r0 + r : nv - 1;
-      }
-      if (d == 0) {
-        for (int comp = 0; comp < 6; comp++)
-#pragma unroll 4
-          for (int loc = lane; loc < Vb; loc += 32) {
-            cplx<float> yv[CC];
-#pragma unroll
-            for (int cc = 0; cc < CC; cc++) yv[cc] = y0[((size_t)cc * 6 + comp) * Vb + loc];
-#pragma unroll
-            for (int r = 0; r < GR; r++) {
-              const float2 pv = __half22float2(Ps[((size_t)ir[r] * 6 + comp) * Vb + loc]);
-#pragma unroll
-              for (int cc = 0; cc < CC; cc++) cmac_conj(acc[r][cc], cplx<float>(pv.x, pv.y), yv[cc]);
-            }
-          }
-      } else {
-        const int k = d - 1;
-        for (int comp = 0; comp < 6; comp++)
-#pragma unroll 2
-          for (int q = f.off[k] + lane; q < f.off[k + 1]; q += 32) {
-            const int fl = f.list[q];
-            cplx<float> yv[CC];
-#pragma unroll
-            for (int cc = 0; cc < CC; cc++) yv[cc] = yf[((size_t)cc * 6 + comp) * nf + q];
-#pragma unroll
-            for (int r = 0; r < GR; r++) {
-              const float2 pv = __half22float2(Ps[((size_t)ir[r] * 6 + comp) * Vb + fl]);
-#pragma unroll
-              for (int cc = 0; cc < CC; cc++) cmac_conj(acc[r][cc], cplx<float>(pv.x, pv.y), yv[cc]);
-            }
-          }
-      }
-#pragma unroll
-      for (int r = 0; r < GR; r++)
-#pragma unroll
-        for (int cc = 0; cc < CC; cc++) {
-          acc[r][cc].re = warp_sum(acc[r][cc].re);
-          acc[r][cc].im = warp_sum(acc[r][cc].im);
-          if (lane == 0 && r0 + r < nv && cc < ncol)
-            Dc[(((size_t)A * 9 + d) * n + col0 + cc) * n + s * nv + r0 + r] = make_float2(acc[r][cc].re, acc[r][cc].im);
-        }
-    }
-    __syncthreads();
-  }
-}
-
 // ---- Galerkin build with matrix instructions -----------------------------------------
 // The same products, for FP16 coarse storage: one CTA per (aggregate A, row chirality s) keeps the nv rows of P on A
 // as FP16 in shared memory and forms, for each part d (self, then the faces) and X sites at a time, the
 // chirality-s components y of all n columns in FP32; their projections are a dense contraction
 //   D[i][j] = sum over (component, site) conj(P_i) y_j
 // done by mma.sync m16n8k8 in TF32: P's FP16 entries are exact in TF32, y goes in as hi + lo (22 bits), and the sums keep
-// what the unit cuts off (mma_sum): 2.5e-8 against 64-bit sums of the same operands (8^4, 24 vectors), the FP32 sums of
-// k_galerkin_rows 4.7e-8, one chain of accumulators 2.3e-5.  (The operands sit in registers and shared memory
+// what the unit cuts off (mma_sum): 2.5e-8 against 64-bit sums of the same operands (8^4, 24 vectors), sums by FP32 lanes
+// and warps 4.7e-8, one chain of accumulators 2.3e-5.  (The operands sit in registers and shared memory
 // where the FP32 stencil leaves them; the contraction is 43 GFLOP at 16^3 x 32, a small part of the time, so the
 // tensor-memory path would not pay for staging operand images.)  16^3 x 32, n = 48: 3.17 ms (2.75 without the cut parts),
-// k_galerkin_rows<2> 6.95 ms (its projections took 17 shared-memory loads per 32 multiply-adds and a warp reduction per
-// entry); what is left is the latency of the P and link loads at 12 warps per SM.  Columns are spread over the threads X
-// sites x (GM_THREADS / X) column groups, GM_CPT columns per thread sharing each link.
+// with FP32 projections out of shared memory 6.95 ms (17 loads per 32 multiply-adds and a warp reduction per entry); what
+// is left is the latency of the P and link loads at 12 warps per SM.  Columns are spread over the threads X sites x
+// (GM_THREADS / X) column groups, GM_CPT columns per thread sharing each link.
 static const int GM_THREADS = 384, GM_CPT = 4;
 
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -512,10 +377,6 @@ static bool try_galerkin_mma(const FineGeom& g, float2* Dc, const float2* P, Lin
   return true;
 }
 
-static size_t galerkin_rows_smem(const FineGeom& g, const FaceDev& faces, int nv, int cc) {
-  return (size_t)nv * 6 * g.Vb * sizeof(__half2) + (size_t)cc * 6 * (g.Vb + faces.off[8]) * sizeof(cplx<float>);
-}
-
 void launch_galerkin(const FineGeom& g, const FaceDev& faces, int dprec, void* Dc, const float2* P, const void* links32,
                      const void* clover32, int nv, bool rows_fp16, cudaStream_t st) {
   ScopedTimer timer_("galerkin", st);
@@ -529,20 +390,15 @@ void launch_galerkin(const FineGeom& g, const FaceDev& faces, int dprec, void* D
   Links<PREC_F32> U{(const float2*)links32, g.Vb};
   Clover<PREC_F32> C{(const float2*)clover32, g.Vb};
   if (dprec != PREC_F32) throw Error(DDTM_ERR_ARG, "internal: Galerkin output is FP32");
-  const size_t srows1 = galerkin_rows_smem(g, faces, nv, 1), srows2 = galerkin_rows_smem(g, faces, nv, 2);
-  // FP16 rows of P where FP16 coarse storage is asked for and they fit in shared memory with the columns of k_galerkin_rows
-  // (4^4 aggregates: up to 30 vectors); beyond that the rows stay FP32 (k_galerkin), although the matrix instructions
-  // would hold two vectors more: FP16 rows there cost D_c another 2e-4.  Widest chunk of sites that fits.
-  const bool rows = rows_fp16 && (srows1 <= 220 * 1024 || srows2 <= 224 * 1024);
-  if (rows && (try_galerkin_mma<32>(g, (float2*)Dc, P, U, C, q, f, nv, st) || try_galerkin_mma<16>(g, (float2*)Dc, P, U, C, q, f, nv, st) ||
-               try_galerkin_mma<8>(g, (float2*)Dc, P, U, C, q, f, nv, st))) {
-  } else if (rows_fp16 && srows2 <= 224 * 1024) {  // two columns per pass where the shared memory holds them
-    set_dynamic_smem((const void*)k_galerkin_rows<2>, srows2);
-    k_galerkin_rows<2><<<g.Nb * 2, threads, srows2, st>>>((float2*)Dc, P, U, C, q, f, nv);
-  } else if (rows_fp16 && srows1 <= 220 * 1024) {
-    set_dynamic_smem((const void*)k_galerkin_rows<1>, srows1);
-    k_galerkin_rows<1><<<g.Nb * 2, threads, srows1, st>>>((float2*)Dc, P, U, C, q, f, nv);
-  } else {
+  // FP16 rows of P where FP16 coarse storage is asked for and they take no more than 220 KB beside one column and its face
+  // hops in FP32 (4^4 aggregates: up to 30 vectors).  Beyond that the rows stay FP32 (k_galerkin), although the
+  // matrix instructions would hold two vectors more: FP16 rows cost D_c 2e-4.  Widest chunk of sites that fits.
+  const size_t rows = (size_t)nv * 6 * g.Vb * sizeof(__half2) + (size_t)6 * (g.Vb + faces.off[8]) * sizeof(cplx<float>);
+  const bool mma = rows_fp16 && rows <= 220 * 1024 &&
+                   (try_galerkin_mma<32>(g, (float2*)Dc, P, U, C, q, f, nv, st) ||
+                    try_galerkin_mma<16>(g, (float2*)Dc, P, U, C, q, f, nv, st) ||
+                    try_galerkin_mma<8>(g, (float2*)Dc, P, U, C, q, f, nv, st));
+  if (!mma) {
     set_dynamic_smem((const void*)k_galerkin<float2>, smem);
     k_galerkin<float2><<<g.Nb, threads, smem, st>>>((float2*)Dc, P, U, C, q, f, nv);
   }
@@ -878,7 +734,7 @@ static void coarse_split_t(const CoarseLevel& c, cplx<float>* y, const cplx<floa
       y, xs, xh, c.Dc.as<float2>(), tab, osite, nout, c.n, c.nv, R, S, H, (float)mu_c, mode, sres, sy, Dinv, rhs, sr);
   CKL("coarse_split");
 }
-// Units of a hop: two on lattices with at most two CTAs per SM, where the chain of a unit's loads is what counts, and one
+// Units of a hop: two on lattices of up to two sites per SM, where the chain of a unit's loads is what counts, and one
 // beyond (2592 sites of 48 dofs, 12 columns: 350 us with one, 388 with two).  Four columns per CTA, fewer where R is 1 or
 // 2 (with 12 columns a matrix entry is loaded once for 12 right-hand sides, but the registers leave too few warps: 421).
 static void coarse_split(const CoarseLevel& c, cplx<float>* y, const cplx<float>* xs, const cplx<float>* xh, const int* tab,
@@ -921,6 +777,8 @@ void launch_coarse_apply_odd(const CoarseLevel& c, cplx<float>* y_o, const cplx<
 void launch_coarse_even(const CoarseLevel& c, cplx<float>* t, const cplx<float>* rhs, const cplx<float>* v, int R, float sr,
                         float sh, cudaStream_t st) {
   ScopedTimer timer_("coarse_even_f32", st, R);
+  // Batches beyond this size are refused, as ever: they never fitted the shared-memory stage of the callers' even-site
+  // kernel.  (k_coarse_split itself stages four columns at a time and would take them.)
   if ((size_t)coarse_shape(c.n, R).spb * c.n * R * sizeof(cplx<float>) > 200 * 1024)
     throw Error(DDTM_ERR_ARG, "coarse_even: " + std::to_string(R) + " right-hand sides of " + std::to_string(c.n) +
                                   " dofs exceed the shared-memory stage");

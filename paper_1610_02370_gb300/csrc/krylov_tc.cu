@@ -12,10 +12,10 @@
 // *err like the tensor-core passes.  Every barrier has a counter of its own, clear when its first CTA arrives: a step
 // clears the counters that its later barriers make free, and the launch of a cycle's first step (no basis vectors) clears all.
 // Bound by reading the basis twice (HBM, or L2 where it fits) and, where it is small, by the latency of three
-// barriers and of the FP64 tail (hence inv_sqrt and the warps that share a tile).  Measured per iteration over a
-// solve, between events: 24^3 x 48, 12 right-hand sides, 59 vectors on average: 69 us; before (multi-dot,
+// barriers and of the FP64 tail (hence inv_sqrt and the warps that share a tile).  Measured per step over a solve with
+// restarts of 100, between events: 24^3 x 48, 12 right-hand sides, 43 vectors on average: 68 us; before (multi-dot,
 // multi-axpy, two reductions, Givens, scaling and image kernels, vectors interleaved by right-hand side) 126 us;
-// 16^3 x 32: 29 us, before 66; 16 x 8^3, one right-hand side: 19 us, before 90.
+// 16^3 x 32, 21 vectors: 30 us, before 66; 16 x 8^3, one right-hand side, 12 vectors: 18 us, before 90.
 // Shapes tried at 24^3 x 48: 4 CTAs of 256 threads per SM 107 us, one of 1024 with 4 vectors in flight 97 us
 // (tiles bunched on some SMs, FP64 sums in the tail); now the fewest warps that cover the tiles, with the registers
 // spent on vectors in flight.

@@ -669,10 +669,10 @@ static void launch_sap_rg(const FineGeom& g, void* x, float* xn, const void* b, 
 }
 
 // Right-hand sides per CTA: up to DDTM_SAP_RG where the batch and the shared memory allow it, fewer
-// otherwise; FP64 keeps one.  Two per CTA (99 KB of FP32 block vectors for 4^4 blocks, 2 CTAs per
-// SM) measured fastest at 32^3 x 64 with 12 and 24 right-hand sides: 34.7 / 68.9 ms per two cycles,
-// against 36.7 / 74.2 ms with one and 37.3 / 73.8 ms with four (whose 198 KB of shared memory leave
-// little L1 for the shared operator data).
+// otherwise; FP64 keeps one.  For blocks other than 4^4; measured on 4^4 blocks before these had kernels of
+// their own: two per CTA (99 KB of FP32 block vectors, 2 CTAs per SM) was fastest at 32^3 x 64 with 12 and 24
+// right-hand sides: 34.7 / 68.9 ms per two cycles, against 36.7 / 74.2 ms with one and 37.3 / 73.8 ms with
+// four (whose 198 KB of shared memory leave little L1 for the shared operator data).
 #ifndef DDTM_SAP_RG
 #define DDTM_SAP_RG 2
 #endif

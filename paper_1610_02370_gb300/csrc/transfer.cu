@@ -104,7 +104,7 @@ __global__ void k_build_P(float2* __restrict__ P, const float2* __restrict__ tv,
   }
 }
 
-// The same orthonormalisation, operation for operation, with the finished vectors kept on chip: the first ns of
+// The same orthonormalisation (its warp sums in another order), with the finished vectors kept on chip: the first ns of
 // them in shared memory, the rest (up to NR) in registers; each thread only ever reads its own site, so the
 // 4 i vector reads that orthogonalising vector i takes never leave the SM.  One CTA of 256 threads per SM.
 // 16^3 x 32, 24 vectors, 4^4 aggregates: 1.73 ms, k_build_P 2.34 ms, which is bound by 14 GB of L2 reads.  Bound by the
